@@ -369,6 +369,10 @@ mrcm_status mrcm_setup(const mrcm_problem* problem, const mrcm_params* params, v
   tab.insert(tab.end(), P.rank.begin(), P.rank.end());
   for (int s = 0; s < P.S; ++s)
     for (int k = 0; k < 4; ++k) tab.push_back(P.rank[6 * s + k] >= 0 ? P.off[s] + P.rank[6 * s + k] : -1);
+  if (tab.size() != plan_table_ints(P)) {   // the workspace reserves exactly that many
+    delete h;
+    return fail(nullptr, MRCM_ERR_INVALID_ARG, "internal: plan tables differ from their reserved size");
+  }
   h->tab_host = tab;
   cudaError_t e = cudaMemcpyAsync(at<int>(h, L.tab), h->tab_host.data(), sizeof(int) * tab.size(), cudaMemcpyHostToDevice, st);
   if (P.mf) {   // multifrontal tables (the host copies live in h->plan)

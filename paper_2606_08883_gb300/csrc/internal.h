@@ -80,6 +80,9 @@ struct Plan {
 // Returns an empty string on success, else the reason the input is invalid.
 std::string make_plan(const mrcm_problem& p, const mrcm_params& q, Plan& plan);
 std::vector<int32_t> export_plan(const Plan& plan);
+// Entries of the plan tables kept on the device: iface[3E], home[2E], off[S], rank[6S], cidx[4S]
+// (cidx: the coupling unknown of each subdomain's side, -1 where it has none)
+inline size_t plan_table_ints(const Plan& P) { return 5 * (size_t)P.E + 11 * (size_t)P.S; }
 
 // ------------------------------------------------------------------------------------------
 // Workspace layout (byte offsets, 256-byte aligned).

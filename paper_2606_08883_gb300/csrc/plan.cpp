@@ -452,8 +452,7 @@ Layout make_layout(const Plan& P, const mrcm_params& q) {
   L.apart = take(8 * (2 * ldh + 3) * ARNOLDI_MAX_BLOCKS);
   L.atot = take(8 * (2 * ldh + 3));
   L.aT = take(8 * ldh * ldh);
-  // device copies of the plan tables: iface[3E], home[2E], off[S], rank[6S], coff[S]
-  L.tab = take(4 * (3 * P.E + E2 + S + 6 * S + S + 16));
+  L.tab = take(4 * plan_table_ints(P));    // device copies of the plan tables
   L.total = o;
   return L;
 }
