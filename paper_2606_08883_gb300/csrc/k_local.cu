@@ -134,14 +134,14 @@ __device__ __forceinline__ void tri_advance(int& i, int& j, int step) {
   }
 }
 
+// FP32 boxes wider than 36 cells (FP64 boxes: k_factor_reg; narrower FP32 boxes: k_factor_sweep).
 // nch = 2: the top and the bottom recursion of the twisted order advance together, one line each
 // per iteration on one half of the CTA (each half with its own working arrays), and the middle line
 // follows; nch = 1: the lines one after the other (boxes too wide for two sets of working arrays).
 // Each line: Schur complement, right-looking Cholesky (the next diagonal's square root is taken by
 // the thread that updates it), L^-1 by elimination on the identity, and S^-1 = L^-T L^-1.  The
 // scaled column of L (Cholesky) and the scaled row of L^-1 are written before the updates that
-// read them (two barriers per column), so every update entry is one FMA: the FP64 pipe, which
-// bounds the FP64 factorisation, does half the work of scaling inside the update.
+// read them (two barriers per column), so every update entry is one FMA.
 template <typename T>
 __global__ void __launch_bounds__(256) k_factor(Geo g, int kind, int LS, T* __restrict__ Linv, int* flags, int nch) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -573,6 +573,170 @@ __global__ void __launch_bounds__(64) k_factor_sweep(Geo g, int kind, int LS, fl
   if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(flags, FLAG_SINGULAR_LOCAL);
 }
 
+// --------------------------------------------------------------------------------------------
+// FP64 factorisation, register-resident: one half of the CTA (FR_HT threads) per recursion of the
+// twisted order, the packed lower triangle of the line block spread over the half's registers
+// (entry t = thread + FR_HT r, so a line is written out coalesced).  Each line: the Schur complement
+// from the previous line's inverse, still in the registers, then w pivots of the symmetric
+// Gauss-Jordan sweep (pivot k: w_i = a_ik / a_kk; a_ij -= w_i a_kj off row and column k, which take
+// w, and a_kk = -1 / a_kk), after which the registers hold -S_J^-1.  A pivot publishes its column
+// and then its scaled column through shared memory, two barriers of the half.
+//
+// The FP64 pipe bounds it: a warp-wide FP64 instruction holds its scheduler's pipe for 64 to 80
+// clocks whatever it computes, so the layout is chosen by the number of such instructions per
+// pivot: npk / 64 rounded up, all lanes busy, plus the reciprocal (three) and the scaling on one
+// warp (36 wide: 13.5 on average; a 128-thread half needs 8.25 on twice the warps, a one-warp half
+// 26, and both lose to it from 256 boxes on).  At most 128 registers are taken up to 40 columns: with
+// four boxes per SM the pipe is 84 % busy, and a wider launch ends in a shorter last wave.  Against
+// one-CTA Cholesky, L^-1 and L^-T L^-1 in shared memory (164 block barriers per line): set-up of
+// 512^2 cells in 40-wide boxes 5.5 -> 3.8 ms, of 1024^2 in 36-wide boxes 17.8 -> 10.0 ms, of 64^2 in
+// 20-wide boxes 0.70 -> 0.48 ms.  Errors against 80-bit solves are 0.8 to 1.0 times those of the
+// Cholesky route (log-normal, channel and white-noise boxes).
+// --------------------------------------------------------------------------------------------
+constexpr int FR_HT = 64;
+
+// 1 / d from the hardware's reciprocal estimate (about 20 bits) by one cubic step,
+// r <- r + r (e + e^2) with e = 1 - d r: three dependent FMAs (within 2.3e-16 of 1 / d).  A result
+// outside the normal range takes the division.
+__device__ __forceinline__ double recip(double d) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
+  const double e = fma(-d, r, 1.0);
+  const double v = fma(r, fma(e, e, e), r);
+  const int ex = __double2hiint(v) & 0x7ff00000;   // integer tests: FP64 compares would take the FP64 pipe
+  return ex != 0 && ex != 0x7ff00000 ? v : 1.0 / d;
+}
+// d > 0 and finite, by its bits
+__device__ __forceinline__ bool positive_finite(double d) {
+  const long long v = __double_as_longlong(d);
+  return v > 0 && v < 0x7ff0000000000000LL;
+}
+
+// Barrier of one half of the CTA
+__device__ __forceinline__ void half_sync(int half) {
+  if (half == 0) asm volatile("bar.sync 1, %0;" ::"n"(FR_HT) : "memory");
+  else asm volatile("bar.sync 2, %0;" ::"n"(FR_HT) : "memory");
+}
+
+template <int WMAX>
+__global__ void __launch_bounds__(2 * FR_HT, WMAX <= 40 ? 4 : 1)
+    k_factor_reg(Geo g, int kind, int LS, double* __restrict__ Linv, int* flags) {
+  static_assert(WMAX <= FR_HT, "one cell of a line per thread");
+  constexpr int NP = WMAX * (WMAX + 1) / 2, R = (NP + FR_HT - 1) / FR_HT, NW = FR_HT / 32;
+  struct Half {
+    double c[2][WMAX + 1];   // pivot column, double-buffered; slot WMAX belongs to the unused entries
+    double w[WMAX + 1];      // the same divided by the pivot
+    double d[WMAX + 1], o[WMAX + 1], e[WMAX + 1];   // the line's diagonal, right and previous-line couplings
+    double r;                // 1 / pivot
+  };
+  __shared__ Half sm_all[2];
+  __shared__ double s_mid[NP];    // the bottom recursion's last S^-1, for the middle line
+  __shared__ double s_e2[WMAX];   // couplings of the middle line to it
+  const int s = blockIdx.x;
+  const bool ohat = kind != BOX_OMEGA_ROBIN, robin = kind != BOX_OHAT_DIRICHLET;
+  const Box b = box_of(g, s, ohat);
+  int rl;
+  const double* rt = robin_tab(g, s, ohat, rl);
+  const int w = b.w, h = b.h, m = h / 2, npk = w * (w + 1) / 2;
+  const int half = threadIdx.x / FR_HT, th = threadIdx.x - half * FR_HT, lane = th & 31, wid = th >> 5;
+  Half& sm = sm_all[half];
+  double* out = Linv + (size_t)s * box_stride(w, h, LS);
+  double* ec_out = out + (size_t)h * LS;
+  double a[R];
+  int ij[R];   // row << 8 | column; unused entries sit in the spare slot WMAX with value 0
+  {
+    int i, j;
+    tri_at(th, i, j);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      ij[r] = th + FR_HT * r < npk ? i << 8 | j : WMAX << 8 | WMAX;
+      a[r] = 0.0;
+      tri_advance(i, j, FR_HT);
+    }
+  }
+  for (int t = th; t <= WMAX; t += FR_HT) sm.c[0][t] = sm.c[1][t] = sm.w[t] = sm.d[t] = sm.o[t] = sm.e[t] = 0.0;
+  bool bad = false;
+  const int nsteps = half == 0 ? m : h - 1 - m;
+  // this thread's cell of the next line: its coefficients are requested one line ahead
+  double pd = 1.0, po = 0.0, pe = 0.0, eprev = 0.0;
+  if (th < w) line_coeffs(g, b, robin, half == 0 ? 0 : h - 1, th, pd, po, pe, rt, rl);
+  for (int it = 0;; ++it) {
+    const bool mid = it == nsteps;
+    if (mid) {   // both recursions are done: the bottom one hands over its last inverse and coupling
+      if (half == 1 && nsteps > 0) {
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+          if (th + FR_HT * r < npk) s_mid[th + FR_HT * r] = -a[r];
+        if (th < w) s_e2[th] = eprev;
+      }
+      __syncthreads();
+      if (half == 1) break;
+    }
+    const int J = half == 0 ? it : h - 1 - it;
+    const bool has_prev = it > 0, dn = mid && m + 1 < h;
+    if (th < w) {
+      sm.d[th] = pd;
+      sm.o[th] = po;
+      sm.e[th] = half == 0 ? pe : eprev;   // towards line J - 1 (top, middle) or J + 1 (bottom)
+      ec_out[(size_t)J * w + th] = pe;
+      eprev = pe;
+      // the next line (the middle one at the latest), in flight over this line's pivots
+      if (!mid) line_coeffs(g, b, robin, half == 0 ? J + 1 : J - 1, th, pd, po, pe, rt, rl);
+    }
+    half_sync(half);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int i = ij[r] >> 8, j = ij[r] & 255;
+      double v = has_prev ? sm.e[i] * a[r] * sm.e[j] : 0.0;   // a = -S_prev^-1
+      if (dn && i < w) v -= s_e2[i] * s_e2[j] * s_mid[th + FR_HT * r];
+      if (i == j) v += sm.d[i];
+      if (i == j + 1) v -= sm.o[j];
+      a[r] = v;
+      if (j == 0) sm.c[0][i] = v;
+    }
+    half_sync(half);
+    for (int k = 0; k < w; ++k) {
+      const double* c = sm.c[k & 1];
+      double* cn = sm.c[(k + 1) & 1];
+      if (wid == k % NW) {   // one warp scales the column, the warps in turn
+        double d = c[k];
+        if (!positive_finite(d)) {
+          bad = true;
+          d = 1.0;
+        }
+        const double ri = recip(d);
+#pragma unroll
+        for (int i0 = 0; i0 < WMAX; i0 += 32)
+          if (i0 + lane < w) sm.w[i0 + lane] = c[i0 + lane] * ri;
+        if (lane == 0) sm.r = ri;
+      }
+      half_sync(half);
+      const double ri = sm.r;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int i = ij[r] >> 8, j = ij[r] & 255;
+        double v = fma(-sm.w[i], c[j], a[r]);
+        if (i == k || j == k) v = i == j ? -ri : sm.w[i == k ? j : i];
+        a[r] = v;
+        if (i == k + 1 || j == k + 1) cn[i == k + 1 ? j : i] = v;
+      }
+      half_sync(half);
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+      if (th + FR_HT * r < npk) out[(size_t)J * LS + th + FR_HT * r] = -a[r];
+    if (mid) break;
+  }
+  if (bad) atomicOr(flags, FLAG_SINGULAR_LOCAL);
+}
+
+template <int WMAX>
+static cudaError_t launch_factor_reg(const Geo& g, int kind, int LS, double* Linv, int* flags, cudaStream_t st) {
+  k_factor_reg<WMAX><<<g.mx * g.my, 2 * FR_HT, 0, st>>>(g, kind, LS, Linv, flags);
+  count_launch(1);
+  return cudaGetLastError();
+}
+
 template <int W>
 static cudaError_t launch_factor_sweep(const Geo& g, int kind, int LS, float* Linv, int* flags, double* coef,
                                        cudaStream_t st) {
@@ -640,10 +804,16 @@ cudaError_t launch_factor(const Geo& g, int kind, int w, int hgt, int LS, void* 
     k_factor<float><<<S, 256, sm, st>>>(g, kind, LS, (float*)Linv, flags, nch);
     count_launch(1);
   } else {
-    const cudaError_t e = raise_smem_limit<k_factor<double>>();
-    if (e != cudaSuccess) return e;
-    k_factor<double><<<S, 256, sm, st>>>(g, kind, LS, (double*)Linv, flags, nch);
-    count_launch(1);
+    double* L = (double*)Linv;
+    if (w <= 16) return launch_factor_reg<16>(g, kind, LS, L, flags, st);
+    if (w <= 20) return launch_factor_reg<20>(g, kind, LS, L, flags, st);
+    if (w <= 24) return launch_factor_reg<24>(g, kind, LS, L, flags, st);
+    if (w <= 28) return launch_factor_reg<28>(g, kind, LS, L, flags, st);
+    if (w <= 32) return launch_factor_reg<32>(g, kind, LS, L, flags, st);
+    if (w <= 36) return launch_factor_reg<36>(g, kind, LS, L, flags, st);
+    if (w <= 40) return launch_factor_reg<40>(g, kind, LS, L, flags, st);
+    if (w <= 48) return launch_factor_reg<48>(g, kind, LS, L, flags, st);
+    return launch_factor_reg<64>(g, kind, LS, L, flags, st);
   }
   return cudaGetLastError();
 }
