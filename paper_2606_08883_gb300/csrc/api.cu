@@ -173,7 +173,6 @@ MfDev mfdev(mrcm_handle h) {
   const Plan& P = h->plan;
   m.fr = at<MfFront>(h, L.mf_fr);
   m.order = at<int>(h, L.mf_ord);
-  m.lvl = at<int>(h, L.mf_lvl);
   m.idx = at<int>(h, L.mf_idx);
   m.asmv = at<int2>(h, L.mf_asm);
   m.map = at<int>(h, L.mf_map);
@@ -181,9 +180,12 @@ MfDev mfdev(mrcm_handle h) {
   m.F = at<double>(h, L.mf_F);
   m.V = at<double>(h, L.mf_V);
   m.scr = at<unsigned>(h, L.mf_scr);
-  m.done = at<unsigned>(h, L.mf_done);
-  m.nfront = (int)P.mf_front.size();
-  m.levels = P.mf_level.empty() ? 0 : (int)P.mf_level.size() - 1;
+  m.item = at<MfItem>(h, L.mf_item);
+  m.inv = at<int2>(h, L.mf_inv);
+  m.rhs = at<int2>(h, L.mf_rhs);
+  m.W = at<uint4>(h, L.mf_msg);
+  m.X = m.W + P.mf_wslots;
+  m.nitem = (int)P.mf_item.size();
   m.max_f = P.mf_max_f;
   m.mcap = P.mf_mcap;
   return m;
@@ -382,13 +384,15 @@ mrcm_status mrcm_setup(const mrcm_problem* problem, const mrcm_params* params, v
     };
     up(L.mf_fr, HP.mf_front.data(), sizeof(MfFront) * HP.mf_front.size());
     up(L.mf_ord, HP.mf_order.data(), 4 * HP.mf_order.size());
-    up(L.mf_lvl, HP.mf_level.data(), 4 * HP.mf_level.size());
     up(L.mf_idx, HP.mf_idx.data(), 4 * HP.mf_idx.size());
     up(L.mf_asm, HP.mf_asm.data(), 4 * HP.mf_asm.size());
     up(L.mf_map, HP.mf_map.data(), 4 * HP.mf_map.size());
     up(L.mf_task, HP.mf_task.data(), 4 * HP.mf_task.size());
+    up(L.mf_item, HP.mf_item.data(), sizeof(MfItem) * HP.mf_item.size());
+    up(L.mf_inv, HP.mf_inv.data(), 4 * HP.mf_inv.size());
+    up(L.mf_rhs, HP.mf_rhs.data(), 4 * HP.mf_rhs.size());
     if (e == cudaSuccess) e = cudaMemsetAsync(h->ws + L.mf_scr, 0, 64, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->ws + L.mf_done, 0, 8 * HP.mf_front.size(), st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(h->ws + L.mf_msg, 0, mf_message_bytes(HP), st);
   }
   if (e == cudaSuccess) e = cudaMemsetAsync(at<unsigned char>(h, L.red), 0, 8 * RED_DOUBLES + 64, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(at<int>(h, L.flags), 0, 4 * 64, st);
@@ -582,7 +586,7 @@ static mrcm_status apply_T(mrcm_handle h, const double* r, double* z, cudaStream
   {
     Phase ph(h, MRCM_PH_COARSE_SOLVE, st);
     if (h->coarse_mf) {
-      CK(h, launch_mf_solve(mfdev(h), c, at<double>(h, L.mom0), P.E, at<int>(h, L.flags), st));
+      CK(h, launch_mf_solve(mfdev(h), at<double>(h, L.mom0), c.g, at<int>(h, L.flags), st));
     } else if (P.NC <= COARSE_DENSE_MAX) {
       CK(h, launch_coarse_apply(c, at<double>(h, L.Ginv), at<double>(h, L.mom0), P.E, st));
     } else {

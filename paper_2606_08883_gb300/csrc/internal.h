@@ -25,16 +25,24 @@ struct MfFront {
   long long fo;   // offset (doubles) of F in the front buffer
   int np, nu;
   int io;         // first of its np + nu unknowns in the index list
-  int vo;         // offset (doubles) of its solve vectors [v_P, w_U]
+  int wo;         // first of its nu slots in the solve's upward messages
   int ao, na;     // its assembly pairs
   int nch;        // children (0..2)
   int ch[2];      // child front ids
   int mo[2];      // offsets of the children's maps
   int par;        // parent front id (-1 at the root)
 };
+// One part of a front in the solve: forward rows [u0, u1) of B, backward rows [p0, p1) of [F11^-1 D];
+// every part of a front forms the whole v_P and keeps it at vo (doubles) of the solve's vectors.
+struct MfItem {
+  int front, u0, u1, p0, p1, vo;
+};
 constexpr int MF_LEAF = 16;       // leaf rectangles of at most this many subdomains
 constexpr int MF_MAX_NP = 128;    // largest pivot block (its inverse is formed in shared memory)
 constexpr int MF_TILE = 32;       // tile of the D, B and S products
+constexpr int MF_PARTS = 304;     // parts per level that the solve aims at (two CTAs on each of 152 SMs)
+constexpr int MF_PART_ROWS = 8;   // rows below which a part is not split further
+constexpr int MF_STAGE = 6144;    // doubles of front rows that a part stages in shared memory
 
 struct Plan {
   int dim = 2;
@@ -71,15 +79,20 @@ struct Plan {
   std::vector<int> mf_task_b;      // [levels + 1] starts of each level's D / B tasks
   std::vector<int> mf_task_c;      // [levels + 1] starts of each level's Schur-complement tasks
   size_t mf_fbuf = 0;              // doubles of all fronts (F and B)
-  size_t mf_vbuf = 0;              // doubles of the solve vectors
+  std::vector<MfItem> mf_item;     // the solve's work, level by level
+  std::vector<int> mf_inv;         // per front position (as mf_idx) the children's message slots, -1 for none
+  std::vector<int> mf_rhs;         // per unknown the two side moments of its right-hand side (~ on the second: subtracted)
+  size_t mf_vbuf = 0;              // doubles of the parts' v_P
+  int mf_wslots = 0;               // upward message slots (sum of nu)
   int mf_max_np = 0, mf_max_f = 0;
-  int mf_mcap = 0;                 // front rows staged by the solve (doubles, padded rows): the largest B or
-                                   // [F11^-1 D], capped at 24576 (192 KB)
+  int mf_mcap = 0;                 // largest staged part (doubles, padded rows), at most MF_STAGE
 };
 
 // Returns an empty string on success, else the reason the input is invalid.
 std::string make_plan(const mrcm_problem& p, const mrcm_params& q, Plan& plan);
 std::vector<int32_t> export_plan(const Plan& plan);
+// bytes of the multifrontal solve's messages: one 16-byte slot per update unknown of a front and per unknown
+inline size_t mf_message_bytes(const Plan& P) { return P.mf ? 16 * ((size_t)P.mf_wslots + P.NC) : 0; }
 // Entries of the plan tables kept on the device: iface[3E], home[2E], off[S], rank[6S], cidx[4S]
 // (cidx: the coupling unknown of each subdomain's side, -1 where it has none)
 inline size_t plan_table_ints(const Plan& P) { return 5 * (size_t)P.E + 11 * (size_t)P.S; }
@@ -98,8 +111,9 @@ struct Layout {
   size_t gtr;                             // Robin coefficients of the Gamma faces, k_local.cu
   size_t rto, rtl;                        // t_R of the Robin box faces of the oversampled / subdomain boxes
   size_t gbML, gbMU, gbX, gbY, gbF, gbC;  // blocked substitution (above COARSE_DENSE_MAX), k_coarse.cu
-  size_t mf_fr, mf_ord, mf_lvl, mf_idx, mf_asm, mf_map, mf_task;   // multifrontal tables, k_mf.cu
-  size_t mf_F, mf_V, mf_scr, mf_done;     // fronts, solve vectors, scratch words, completion flags
+  size_t mf_fr, mf_ord, mf_idx, mf_asm, mf_map, mf_task;   // multifrontal tables, k_mf.cu
+  size_t mf_item, mf_inv, mf_rhs;         // its solve's work list, message slots and right-hand sides
+  size_t mf_F, mf_V, mf_scr, mf_msg;      // fronts, solve vectors, scratch words, messages (upward, then x)
   size_t rho, zt;                         // FP32 staged right-hand sides (k_stage32), apply output scratch
   size_t V, Z, w, Hs, red, flags, tmpv;   // Krylov basis and scratch
   size_t tab;                             // device copies of the plan tables
@@ -313,18 +327,20 @@ cudaError_t launch_coarse_apply(const CoarseDev& c, const double* Ginv, const do
 struct MfDev {
   const MfFront* fr;
   const int* order;
-  const int* lvl;       // [levels + 1]
   const int* idx;
   const int2* asmv;
   const int* map;
   const int4* task;
+  const MfItem* item;   // [nitem] the solve's parts, level by level
+  const int2* inv;      // message slots of each front position's children (-1: none)
+  const int2* rhs;      // side moments of each unknown's right-hand side
   double* F;
-  double* V;
+  double* V;            // the parts' v_P
+  uint4* W;             // upward messages (w_U of every front)
+  uint4* X;             // solution entries as messages [2E nq]
   unsigned* scr;        // [2, 6) two 8-byte maxima (|G| entries, |S| entries); [8] solve epoch,
                         // [9] CTAs finished in the current solve
-  unsigned* done;       // [2 nfront] forward / backward completion epochs of each front
-  int levels;
-  int nfront;
+  int nitem;
   int max_f;            // largest front (np + nu)
   int mcap;             // doubles of front rows the solve stages in shared memory
 };
@@ -333,11 +349,9 @@ struct MfDev {
 // when a pivot is zero or not finite or |S| grows past NOPIV_MAX_GROWTH max |G| (the caller then
 // falls back to the pivoted band LU).
 cudaError_t launch_mf_factor(const MfDev& m, const Plan& P, const double* ab, int* flags, cudaStream_t st);
-// Per apply: right-hand side from mom0 (through c), then one cooperative launch: forward through
-// the levels, backward down them, each front waiting on its children's (parent's) completion
-// flags; the solution replaces c.g.
-cudaError_t launch_mf_solve(const MfDev& m, const CoarseDev& c, const double* mom0, int E, int* flags,
-                            cudaStream_t st);
+// Per apply, one cooperative launch: right-hand side from mom0, forward through the levels and
+// backward down them, every part of a front polling the entries that it needs; the solution goes to g.
+cudaError_t launch_mf_solve(const MfDev& m, const double* mom0, double* g, int* flags, cudaStream_t st);
 cudaError_t launch_arnoldi(const Geo& g, const double* z, double* V, int j, size_t n, double* H, int ldh, double* cs,
                            double* sn, double* gv, double* out, double* wbuf, double* part, double* tot, double* Tm,
                            unsigned* bar, int* flags, cudaStream_t st);

@@ -358,13 +358,13 @@ cudaError_t launch_mf_factor(const MfDev& m, const Plan& P, const double* ab, in
 }
 
 // y_r = sum_k A[r][k] x[k] for r < rows (A row-major with leading dimension lda, in shared or global
-// memory): tpr threads per row (a power of two up to 8, as many as the CTA has for the rows), each
+// memory): tpr threads per row (a power of two up to a warp, as many as the CTA has for the rows), each
 // with four partial sums over its columns k = q, q + tpr, ..., then the tpr sums in a fixed shuffle
 // order; emit(r, y) by the first thread of the row.  Deterministic.
 template <class Emit>
 __device__ __forceinline__ void mf_rows(const double* A, int lda, int rows, int cols, const double* x, Emit emit) {
   int tpr = 1;
-  while (tpr < 8 && tpr * 2 * rows <= MF_THREADS) tpr *= 2;
+  while (tpr < 32 && tpr * 2 * rows <= MF_THREADS) tpr *= 2;
   const int q = threadIdx.x % tpr, per = MF_THREADS / tpr;
   for (int r0 = 0; r0 < rows; r0 += per) {
     const int r = r0 + threadIdx.x / tpr;
@@ -395,125 +395,104 @@ __device__ __forceinline__ void cp_async_wait_all() {
   asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
 }
 
-// Solve, one cooperative launch (one CTA per SM), fronts taken level by level in round robin: a
-// front's forward step waits for its children's, its backward step for its parent's (the
-// ancestors have then written x_U), through completion flags stamped with the solve's epoch.  The
-// epoch lives in device memory: every CTA reads it at the start, the last CTA to finish advances
-// it, so repeated launches (also from a captured graph) never see a stale flag as current.  All
-// CTAs are resident and each takes its fronts in increasing level (decreasing, backward), so
-// every wait ends; the spins are bounded all the same (FLAG_TIMEOUT).  Everything a step reads
-// that does not depend on the wait (the front's indices, its right-hand side entries, its B or
-// [F11^-1 D] rows, copied asynchronously into shared memory) is requested before the wait, so a
-// level costs about one flag hand-over and one read.  A front's rows are dotted by whole warps
-// (up to eight threads per row, four partial sums each, combined in a fixed order), so the result
-// is deterministic.
-__global__ void __launch_bounds__(MF_THREADS) k_mf_solve(MfDev m, double* __restrict__ g, int* flags, int mcap) {
+// Messages: a double in a 16-byte slot as two (half, epoch) pairs.  Each 8-byte pair is written and
+// read at once, so a slot whose two epochs are the solve's holds the solve's value, and no fence or
+// separate flag is needed.
+__device__ __forceinline__ void msg_put(uint4* slot, double v, unsigned E) {
+  asm volatile("st.volatile.global.v4.u32 [%0], {%1, %2, %3, %4};\n" ::"l"(slot), "r"((unsigned)__double2loint(v)), "r"(E),
+               "r"((unsigned)__double2hiint(v)), "r"(E)
+               : "memory");
+}
+// Polls a slot.  The wait is bounded: when it gives up, here or in any other CTA (FLAG_TIMEOUT is set),
+// it returns 0 and the later waits of the launch give up after a few polls.
+__device__ __forceinline__ double msg_get(const uint4* slot, unsigned E, int* flags) {
+  for (long long spins = 0; spins < BARRIER_SPIN_LIMIT; ++spins) {
+    unsigned lo, e0, hi, e1;
+    asm volatile("ld.volatile.global.v4.u32 {%0, %1, %2, %3}, [%4];\n"
+                 : "=r"(lo), "=r"(e0), "=r"(hi), "=r"(e1)
+                 : "l"(slot)
+                 : "memory");
+    if (e0 == E && e1 == E) return __hiloint2double((int)hi, (int)lo);
+    if ((spins & 1023) == 1023 && (*(volatile int*)flags & FLAG_TIMEOUT)) return 0.0;
+  }
+  atomicOr(flags, FLAG_TIMEOUT);
+  return 0.0;
+}
+
+// Solve, one cooperative launch.  A part of a front takes its rows forward (w_U = v_U - B v_P, with
+// v_P = g_P + the children's w, v_U their part mapped into U) and backward (x_P = F11^-1 v_P - D x_U);
+// it polls the entries that it needs from the children's parts, or of x from the ancestors', each entry
+// carrying the solve's epoch.  The epoch lives in device memory: every CTA reads it at the start, the
+// last CTA to finish advances it, so repeated launches (also from a captured graph) never take an old
+// entry for a current one.  All CTAs are resident, and each takes its parts in increasing level
+// (decreasing, backward), so every wait ends; the waits are bounded all the same.  What a part reads
+// besides (its rows of B or [F11^-1 D], copied into shared memory, its slots) is requested before it
+// waits.  Rows are dotted by up to a warp each, in a fixed order, so the result is deterministic.
+//
+// The dependence chain bounds it: 2 x levels hand-overs, each a write, a poll and a short product.  With
+// the whole front on one CTA the upper levels' products alone took 2.4 to 4.7 us there (128 x 128 FMA at
+// 1.6 a clock), and a completion flag per front cost a fence, a poll by one thread and a second read:
+// 131 us on 64 x 64 subdomains (9 levels), 80 us on 32 x 32, 56 us on 16 x 16, with the right-hand side
+// formed by a launch of its own; now 60, 39 and 25 us.
+__global__ void __launch_bounds__(MF_THREADS, 2) k_mf_solve(MfDev m, const double* __restrict__ mom0,
+                                                         double* __restrict__ g, int* flags, int mcap) {
   extern __shared__ __align__(16) double smd[];
-  double* v = smd;                                   // [max_f]
-  double* M = v + m.max_f;                           // [mcap] rows of B or of [F11^-1 D]
-  int* ix = reinterpret_cast<int*>(M + mcap);        // [max_f]
-  __shared__ unsigned s_ep;
-  __shared__ int s_ok;
+  double* v = smd;           // [max_f]
+  double* M = v + m.max_f;   // [mcap] rows of B or of [F11^-1 D], with an odd stride
   volatile unsigned* vep = m.scr + 8;
-  if (threadIdx.x == 0) {
-    s_ep = *vep + 1u;
-    s_ok = 1;
-  }
-  __syncthreads();
-  const unsigned E = s_ep;
-  volatile unsigned* fdone = m.done;
-  volatile unsigned* bdone = m.done + m.nfront;
-  // thread 0 polls the flag; the CTA proceeds together (false: the wait gave up)
-  auto wait_for = [&](volatile unsigned* fl) -> bool {
-    if (threadIdx.x == 0) {
-      long long spins = 0;
-      while (*fl != E) {
-        if (++spins > BARRIER_SPIN_LIMIT) {
-          atomicOr(flags, FLAG_TIMEOUT);
-          s_ok = 0;
-          break;
-        }
-      }
-      __threadfence();
-    }
-    __syncthreads();
-    return s_ok != 0;
+  const unsigned E = *vep + 1u;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  auto stage = [&](const double* A, int rows, int cols) -> bool {   // rows x cols, contiguous rows of A
+    if (rows * (cols + 1) > mcap) return false;
+    for (int r = wid; r < rows; r += MF_THREADS / 32)
+      for (int k = lane; k < cols; k += 32) cp_async8(M + (size_t)r * (cols + 1) + k, A + (size_t)r * cols + k);
+    return true;
   };
-  auto publish = [&](volatile unsigned* fl) {
-    __threadfence();
+  const int last = m.nitem - 1 - (m.nitem - 1 - (int)blockIdx.x) % (int)gridDim.x;
+  for (int it = blockIdx.x; it < m.nitem; it += gridDim.x) {
+    const MfItem w = m.item[it];
+    const MfFront fr = m.fr[w.front];
+    const int np = fr.np, f = fr.np + fr.nu, rows = w.u1 - w.u0;
+    const double* Bx = m.F + fr.fo + (size_t)f * f + (size_t)w.u0 * np;
+    const bool staged = stage(Bx, rows, np);
+    for (int t = tid; t < np + rows; t += MF_THREADS) {
+      const int pos = fr.io + (t < np ? t : t + w.u0);
+      const int2 slot = m.inv[pos];
+      double val = 0.0;
+      if (t < np) {
+        const int2 o = m.rhs[m.idx[pos]];
+        val = o.y >= 0 ? -(mom0[o.x] + mom0[o.y]) : -(mom0[o.x] - mom0[~o.y]);
+      }
+      if (slot.x >= 0) val += msg_get(m.W + slot.x, E, flags);
+      if (slot.y >= 0) val += msg_get(m.W + slot.y, E, flags);
+      v[t] = val;
+      if (t < np) m.V[w.vo + t] = val;
+    }
+    cp_async_wait_all();
     __syncthreads();
-    if (threadIdx.x == 0) *fl = E;
-  };
-  bool ok = true;
-  // forward: v_P = g_P + the children's w mapped into P, v_U = their part mapped into U;
-  // keep v_P, pass w_U = v_U - B v_P up
-  for (int L = 0; L < m.levels && ok; ++L) {
-    for (int b = m.lvl[L] + blockIdx.x; b < m.lvl[L + 1] && ok; b += gridDim.x) {
-      const int fid = m.order[b];
-      const MfFront fr = m.fr[fid];
-      const int np = fr.np, nu = fr.nu, f = np + nu;
-      const double* Bx = m.F + fr.fo + (size_t)f * f;
-      // B staged row by row with an odd stride in doubles (np + 1): the rows a warp reads start in
-      // different banks
-      const bool staged = nu * (np + 1) <= mcap;
-      if (staged)
-        for (int r = threadIdx.x >> 5; r < nu; r += MF_THREADS / 32)
-          for (int k = threadIdx.x & 31; k < np; k += 32) cp_async8(M + (size_t)r * (np + 1) + k, Bx + (size_t)r * np + k);
-      for (int t = threadIdx.x; t < f; t += MF_THREADS) v[t] = t < np ? g[m.idx[fr.io + t]] : 0.0;
-      __syncthreads();
-      for (int c = 0; c < fr.nch && ok; ++c) {
-        const int cid = c == 0 ? fr.ch[0] : fr.ch[1];
-        const MfFront cf = m.fr[cid];
-        const int* mp = m.map + (c == 0 ? fr.mo[0] : fr.mo[1]);
-        const double* wc = m.V + cf.vo + cf.np;
-        ok = wait_for(fdone + cid);
-        if (!ok) break;
-        for (int t = threadIdx.x; t < cf.nu; t += MF_THREADS) v[mp[t]] += __ldcg(wc + t);
-        __syncthreads();
-      }
-      if (!ok) break;
-      cp_async_wait_all();
-      __syncthreads();
-      double* Vf = m.V + fr.vo;
-      for (int t = threadIdx.x; t < np; t += MF_THREADS) Vf[t] = v[t];
-      mf_rows(staged ? M : Bx, staged ? np + 1 : np, nu, np, v,
-              [&](int r, double t) { Vf[np + r] = v[np + r] - t; });
-      publish(fdone + fid);
-    }
+    mf_rows(staged ? M : Bx, staged ? np + 1 : np, rows, np, v,
+            [&](int r, double t) { msg_put(m.W + fr.wo + w.u0 + r, v[np + r] - t, E); });
+    __syncthreads();
   }
-  // backward: x_P = [F11^-1 D] [v_P; -x_U], x_U written by the ancestors
-  for (int L = m.levels - 1; L >= 0 && ok; --L) {
-    for (int b = m.lvl[L] + blockIdx.x; b < m.lvl[L + 1] && ok; b += gridDim.x) {
-      const int fid = m.order[b];
-      const MfFront fr = m.fr[fid];
-      const int np = fr.np, nu = fr.nu, f = np + nu;
-      const double* F = m.F + fr.fo;
-      const double* Vf = m.V + fr.vo;
-      const bool staged = np * (f + 1) <= mcap;   // [F11^-1 D], rows with stride f + 1
-      if (staged)
-        for (int r = threadIdx.x >> 5; r < np; r += MF_THREADS / 32)
-          for (int k = threadIdx.x & 31; k < f; k += 32) cp_async8(M + (size_t)r * (f + 1) + k, F + (size_t)r * f + k);
-      for (int t = threadIdx.x; t < f; t += MF_THREADS) {
-        ix[t] = m.idx[fr.io + t];
-        if (t < np) v[t] = Vf[t];
-      }
-      if (fr.par >= 0) {
-        ok = wait_for(bdone + fr.par);
-        if (!ok) break;
-      } else {
-        __syncthreads();
-      }
-      for (int t = np + threadIdx.x; t < f; t += MF_THREADS) v[t] = -__ldcg(g + ix[t]);
-      cp_async_wait_all();
-      __syncthreads();
-      mf_rows(staged ? M : F, staged ? f + 1 : f, np, f, v, [&](int r, double t) { g[ix[r]] = t; });
-      publish(bdone + fid);
-    }
+  for (int it = last; it >= 0; it -= gridDim.x) {
+    const MfItem w = m.item[it];
+    const MfFront fr = m.fr[w.front];
+    const int np = fr.np, f = fr.np + fr.nu, rows = w.p1 - w.p0;
+    const double* F = m.F + fr.fo + (size_t)w.p0 * f;
+    const bool staged = stage(F, rows, f);
+    for (int t = tid; t < f; t += MF_THREADS)
+      v[t] = t < np ? m.V[w.vo + t] : -msg_get(m.X + m.idx[fr.io + t], E, flags);
+    cp_async_wait_all();
+    __syncthreads();
+    mf_rows(staged ? M : F, staged ? f + 1 : f, rows, f, v, [&](int r, double t) {
+      const int u = m.idx[fr.io + w.p0 + r];
+      msg_put(m.X + u, t, E);
+      g[u] = t;
+    });
+    __syncthreads();
   }
   // the last CTA to finish advances the epoch (a CTA that gave up still counts itself)
-  cp_async_wait_all();
-  __syncthreads();
-  if (threadIdx.x == 0) {
+  if (tid == 0) {
     __threadfence();
     if (atomicAdd(m.scr + 9, 1u) == gridDim.x - 1) {
       m.scr[9] = 0u;
@@ -523,24 +502,22 @@ __global__ void __launch_bounds__(MF_THREADS) k_mf_solve(MfDev m, double* __rest
   }
 }
 
-cudaError_t launch_mf_solve(const MfDev& m, const CoarseDev& c, const double* mom0, int E, int* flags,
-                            cudaStream_t st) {
-  cudaError_t e = launch_coarse_rhs(c, mom0, E, st);
+cudaError_t launch_mf_solve(const MfDev& m, const double* mom0, double* g, int* flags, cudaStream_t st) {
+  static const int sms = [] {
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) n = 0;
+    return n;
+  }();
+  cudaError_t e = raise_smem_limit<k_mf_solve>();
   if (e != cudaSuccess) return e;
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  // shared memory: v and the indices of the largest front, and its matrix rows when they fit in
-  // about 192 KB (larger fronts read them from global memory)
-  int mcap = m.mcap;
-  const size_t sm = 12 * (size_t)m.max_f + 8 * (size_t)mcap;
-  e = raise_smem_limit<k_mf_solve>();
-  if (e != cudaSuccess) return e;
+  // v and the staged rows: about 50 KB, so two CTAs fit an SM (one if the largest front is very wide)
+  const size_t sm = 8 * ((size_t)m.max_f + (size_t)m.mcap);
+  const int per_sm = sm <= 112 * 1024 ? 2 : 1;
   MfDev mm = m;
-  double* g = c.g;
-  int* fl = flags;
-  void* args[] = {(void*)&mm, (void*)&g, (void*)&fl, (void*)&mcap};
-  e = cudaLaunchCooperativeKernel((const void*)k_mf_solve, dim3(sms), dim3(MF_THREADS), args, sm, st);
+  int mcap = m.mcap;
+  void* args[] = {(void*)&mm, (void*)&mom0, (void*)&g, (void*)&flags, (void*)&mcap};
+  const int grid = m.nitem < per_sm * sms ? m.nitem : per_sm * sms;
+  e = cudaLaunchCooperativeKernel((const void*)k_mf_solve, dim3(grid), dim3(MF_THREADS), args, sm, st);
   count_launch(1);
   return e;
 }

@@ -143,6 +143,9 @@ std::string make_plan(const mrcm_problem& p, const mrcm_params& q, Plan& P) {
     P.mf_asm.clear();
     P.mf_map.clear();
     P.mf_task.clear();
+    P.mf_item.clear();
+    P.mf_inv.clear();
+    P.mf_rhs.clear();
     P.mf_fbuf = P.mf_vbuf = 0;
   }
   return std::string();
@@ -246,8 +249,10 @@ static bool plan_mf(Plan& P) {
   std::vector<int> pos(P.NC, -1);
   P.mf_asm.clear();
   P.mf_map.clear();
-  size_t fo = 0, vo = 0;
-  P.mf_max_np = P.mf_max_f = P.mf_mcap = 0;
+  size_t fo = 0;
+  int wo = 0;
+  P.mf_max_np = P.mf_max_f = 0;
+  P.mf_inv.assign(2 * P.mf_idx.size(), -1);
   for (int f = 0; f < nf; ++f) {
     MfFront& fr = P.mf_front[f];
     const int fs = fr.np + fr.nu;
@@ -268,20 +273,19 @@ static bool plan_mf(Plan& P) {
         const int p = pos[P.mf_idx[cf.io + cf.np + t]];
         if (p < 0) return false;
         P.mf_map.push_back(p);
+        P.mf_inv[2 * (size_t)(fr.io + p) + c] = cf.wo + t;
       }
     }
     for (int t = 0; t < fs; ++t) pos[P.mf_idx[fr.io + t]] = -1;
     fr.fo = (long long)fo;
     fo += (size_t)fs * fs + (size_t)fr.nu * fr.np;
-    fr.vo = (int)vo;
-    vo += fs;
+    fr.wo = wo;
+    wo += fr.nu;
     P.mf_max_np = std::max(P.mf_max_np, fr.np);
     P.mf_max_f = std::max(P.mf_max_f, fs);
-    P.mf_mcap = std::max(P.mf_mcap, std::min(24576, std::max(fr.np * (fs + 1), fr.nu * (fr.np + 1))));
   }
-  if (vo > (size_t)INT32_MAX) return false;
   P.mf_fbuf = fo;
-  P.mf_vbuf = vo;
+  P.mf_wslots = wo;
   // levels and the tile tasks of each level
   const int nl = *std::max_element(level.begin(), level.end()) + 1;
   P.mf_level.assign(nl + 1, 0);
@@ -312,6 +316,44 @@ static bool plan_mf(Plan& P) {
     }
   }
   P.mf_level[nl] = (int)P.mf_order.size();
+  // the solve's work: each level's fronts cut into parts of rows, so that the few large fronts of the
+  // upper levels are spread over the GPU too, and a part's rows fit its staging buffer
+  size_t vo = 0;
+  P.mf_item.clear();
+  P.mf_mcap = 0;
+  for (int L = 0; L < nl; ++L)
+    for (int i = P.mf_level[L]; i < P.mf_level[L + 1]; ++i) {
+      const MfFront& fr = P.mf_front[P.mf_order[i]];
+      const int f = fr.np + fr.nu, rows = std::max(fr.np, fr.nu);
+      auto staged = [&](int parts) {
+        return std::max((fr.np + parts - 1) / parts * (f + 1), (fr.nu + parts - 1) / parts * (fr.np + 1));
+      };
+      int parts = std::max(1, std::min(MF_PARTS / (P.mf_level[L + 1] - P.mf_level[L]),
+                                       (rows + MF_PART_ROWS - 1) / MF_PART_ROWS));
+      while (parts < rows && staged(parts) > MF_STAGE) ++parts;
+      for (int k = 0; k < parts; ++k) {
+        P.mf_item.push_back({P.mf_order[i], fr.nu * k / parts, fr.nu * (k + 1) / parts, fr.np * k / parts,
+                             fr.np * (k + 1) / parts, (int)vo});
+        vo += fr.np;
+      }
+      P.mf_mcap = std::max(P.mf_mcap, std::min(MF_STAGE, staged(parts)));
+    }
+  if (vo > (size_t)INT32_MAX) return false;
+  P.mf_vbuf = vo;
+  // right-hand side of each unknown's row, -(F_s + F_s') or -(P_s - P_s') of its interface, as offsets
+  // into the particular side moments [S][4 sides][nq tests][F, |f|P]
+  P.mf_rhs.assign(2 * (size_t)P.NC, 0);
+  for (int e = 0; e < P.E; ++e) {
+    const int a = P.iface[3 * e], s = P.iface[3 * e + 1], s2 = P.iface[3 * e + 2];
+    for (int qt = 0; qt < nq; ++qt) {
+      const int m1 = ((s * 4 + 2 * a + 1) * nq + qt) * 2, m2 = ((s2 * 4 + 2 * a) * nq + qt) * 2;
+      const int rf = P.row_home[2 * e] * nq + qt, rp = P.row_home[2 * e + 1] * nq + qt;
+      P.mf_rhs[2 * (size_t)rf] = m1;
+      P.mf_rhs[2 * (size_t)rf + 1] = m2;
+      P.mf_rhs[2 * (size_t)rp] = m1 + 1;
+      P.mf_rhs[2 * (size_t)rp + 1] = ~(m2 + 1);
+    }
+  }
   P.mf_task_b[nl] = P.mf_task_c[nl] = (int)P.mf_task.size() / 4;
   // B and C task starts: a level's S tasks follow its D / B tasks, so the B range of level L is
   // [task_b[L], task_c[L]) and the C range [task_c[L], task_b[L + 1])
@@ -430,15 +472,17 @@ Layout make_layout(const Plan& P, const mrcm_params& q) {
   // multifrontal factorisation of G (k_mf.cu): tables, fronts, solve vectors, scratch words
   L.mf_fr = take(sizeof(MfFront) * P.mf_front.size());
   L.mf_ord = take(4 * P.mf_order.size());
-  L.mf_lvl = take(4 * P.mf_level.size());
   L.mf_idx = take(4 * P.mf_idx.size());
   L.mf_asm = take(4 * P.mf_asm.size());
   L.mf_map = take(4 * P.mf_map.size());
   L.mf_task = take(4 * P.mf_task.size());
   L.mf_F = take(8 * P.mf_fbuf);
+  L.mf_item = take(sizeof(MfItem) * P.mf_item.size());
+  L.mf_inv = take(4 * P.mf_inv.size());
+  L.mf_rhs = take(4 * P.mf_rhs.size());
   L.mf_V = take(8 * P.mf_vbuf);
   L.mf_scr = take(64);
-  L.mf_done = take(8 * P.mf_front.size());
+  L.mf_msg = take(mf_message_bytes(P));
   L.rho = take(8 * n);                     // FP32 right-hand sides staged on the grid (k_stage32)
   L.zt = take(8 * n);
   L.V = take(8 * (size_t)(L.m + 1) * n);
