@@ -91,6 +91,89 @@ __device__ __forceinline__ double robin_tr(double k_in, double k_out, double are
   return 1.0 / (1.0 / tau + beta / area);
 }
 
+// The five-point operator (A v)_c = sum over the four faces of T_f (v_c - v_c') (no flow into cells outside
+// the grid, whose v is 0: a boundary face contributes T_f v_c), applied by a march down columns: a warp
+// takes 31 columns (its first lane holds the column to their left) and the rows [j0, j1), and each face
+// difference is formed once, for the cell on either side of it: the x difference goes to the next lane
+// by a shuffle, the y difference is kept for the next row.  emit(cell, base, s) gets, for each cell, the
+// face sum folded into base(cell) as base + sign * A v, in the order east, west, north, south.
+//
+// Bound by the FP64 pipe (1.6 operations a clock and SM), so what counts is FP64 instructions per cell:
+// two subtractions and four FMAs here, against four and five with every cell forming its own four
+// differences.  2048^2 cells: 73.8 -> 57.4 us (51 at the pipe's rate, 20 of HBM traffic).
+// Rows come in groups of STENCIL_ROWS whose loads are all in flight together.
+constexpr int STENCIL_ROWS = 4;
+constexpr int STENCIL_COLS = 31;
+
+template <int SIGN, class Base, class Emit>
+__device__ __forceinline__ void stencil_march(const Geo& g, const double* __restrict__ v, int col0, int j0, int j1,
+                                              Base base, Emit emit) {
+  const int lane = threadIdx.x & 31, i = col0 + lane - 1;
+  const bool in = i >= 0 && i < g.nx, own = in && lane > 0;
+  auto at = [&](int j) { return in && j >= 0 && j < g.ny ? v[(size_t)j * g.nx + i] : 0.0; };
+  double vc = at(j0), ds = at(j0 - 1) - vc, Ts = own ? g.Ty[(size_t)j0 * g.nx + i] : 0.0;
+  for (int j = j0; j < j1; j += STENCIL_ROWS) {
+    double vn[STENCIL_ROWS], vr[STENCIL_ROWS], Tw[STENCIL_ROWS], Te[STENCIL_ROWS], Tn[STENCIL_ROWS], b[STENCIL_ROWS];
+#pragma unroll
+    for (int q = 0; q < STENCIL_ROWS; ++q) {
+      const bool on = own && j + q < j1;
+      vn[q] = j + q < j1 ? at(j + q + 1) : 0.0;
+      vr[q] = on && lane == 31 && i + 1 < g.nx ? v[(size_t)(j + q) * g.nx + i + 1] : 0.0;
+      const double* Tx = g.Tx + (size_t)(j + q) * (g.nx + 1) + i;
+      Tw[q] = on ? Tx[0] : 0.0;
+      Te[q] = on ? Tx[1] : 0.0;
+      Tn[q] = on ? g.Ty[(size_t)(j + q + 1) * g.nx + i] : 0.0;
+      b[q] = on ? base((size_t)(j + q) * g.nx + i) : 0.0;
+    }
+#pragma unroll
+    for (int q = 0; q < STENCIL_ROWS; ++q) {
+      const double right = __shfl_down_sync(0xffffffffu, vc, 1);
+      const double de = vc - (lane == 31 ? vr[q] : right);
+      const double dw = __shfl_up_sync(0xffffffffu, de, 1);   // v_west - v_c
+      const double dn = vc - vn[q];
+      double s = fma(SIGN * Te[q], de, b[q]);
+      s = fma(-SIGN * Tw[q], dw, s);
+      s = fma(SIGN * Tn[q], dn, s);
+      s = fma(-SIGN * Ts, ds, s);
+      if (own && j + q < j1) emit((size_t)(j + q) * g.nx + i, s);
+      ds = dn;
+      vc = vn[q];
+      Ts = Tn[q];
+    }
+  }
+}
+// The same for one cell alone, base + SIGN A v in the same order (bit for bit the march's)
+template <int SIGN>
+__device__ __forceinline__ double face_sum(const Geo& g, const double* __restrict__ v, int i, int j, double base) {
+  const size_t c = (size_t)j * g.nx + i;
+  const double vc = v[c];
+  const double vw = i > 0 ? v[c - 1] : 0.0;
+  const double ve = i < g.nx - 1 ? v[c + 1] : 0.0;
+  const double vs = j > 0 ? v[c - g.nx] : 0.0;
+  const double vn = j < g.ny - 1 ? v[c + g.nx] : 0.0;
+  const double* Tx = g.Tx + (size_t)j * (g.nx + 1) + i;
+  const double* Ty = g.Ty + c;
+  double s = fma(SIGN * Tx[1], vc - ve, base);
+  s = fma(SIGN * Tx[0], vc - vw, s);
+  s = fma(SIGN * Ty[g.nx], vc - vn, s);
+  return fma(SIGN * Ty[0], vc - vs, s);
+}
+__device__ __forceinline__ double apply_A(const Geo& g, const double* __restrict__ v, int i, int j) {
+  return face_sum<1>(g, v, i, j, 0.0);
+}
+
+// Launch shape of a kernel of 128-thread blocks that march `rows` rows per warp (blockIdx.y).  Long marches
+// where they still give every SM a dozen warps (2 M cells), short ones below, and none (one thread per
+// cell, apply_A) below half a million cells, where a launch is bound by latency: there a march of 16 or
+// 4 rows took 2 to 4 us more than a thread per cell (two launches at 512^2: 21.3 against 17.3 us).
+inline bool stencil_marches(int nx, int ny) { return (size_t)nx * ny >= (size_t)1 << 19; }
+inline int stencil_rows(int nx, int ny) { return (size_t)nx * ny >= (size_t)1 << 21 ? 16 : STENCIL_ROWS; }
+inline dim3 stencil_grid(int nx, int ny) {
+  const int cols = 4 * STENCIL_COLS, rows = stencil_rows(nx, ny);
+  return dim3((nx + cols - 1) / cols, (ny + rows - 1) / rows);
+}
+__device__ __forceinline__ int stencil_col0() { return (blockIdx.x * 4 + (threadIdx.x >> 5)) * STENCIL_COLS; }
+
 // Grid-wide barrier for cooperative launches (every block co-resident).  bar[0] counts arrivals
 // (zero between barriers), bar[1] is the generation.  A block that polls more than
 // BARRIER_SPIN_LIMIT times sets FLAG_TIMEOUT in *flags and returns false instead of waiting on.

@@ -248,7 +248,6 @@ void set_thread_error(const std::string& msg);
 cudaError_t launch_assemble(const Geo& g, const int* bc_kind, const double* const* bcv, const double* f,
                             double* Tx, double* Ty, double* b, cudaStream_t st);
 cudaError_t launch_matvec(const Geo& g, const double* v, double* w, cudaStream_t st);
-cudaError_t launch_residual(const Geo& g, const double* r, const double* z, double* rho, cudaStream_t st);
 // FP64 FMA throughput probe (k_grid.cu): blocks x threads x iters x 32 FMA
 cudaError_t launch_dfma_probe(double* sink, int blocks, int threads, int iters, cudaStream_t st);
 cudaError_t launch_fluxes(const Geo& g, const int* bc_kind, const double* const* bcv, const double* p,

@@ -1,5 +1,5 @@
-// Fine-grid kernels (Sec. 3): face transmissibilities and b, the matrix-free operator A v, the
-// residual r - A z and the face velocities.  Two-point flux form of the statically condensed RT0
+// Fine-grid kernels (Sec. 3): face transmissibilities and b, the matrix-free operator A v and
+// the face velocities.  Two-point flux form of the statically condensed RT0
 // system; 2-D, cells x-fastest, one thread per cell or face, coalesced along x.
 #include "common.cuh"
 
@@ -67,33 +67,14 @@ __global__ void k_rhs(Geo g, BcDev bc, const double* f, double* b) {
   b[c] = v;
 }
 
-__device__ __forceinline__ double apply_A(const Geo& g, const double* __restrict__ v, int i, int j) {
-  const size_t c = (size_t)j * g.nx + i;
-  const double vc = v[c];
-  const double vw = i > 0 ? v[c - 1] : 0.0;
-  const double ve = i < g.nx - 1 ? v[c + 1] : 0.0;
-  const double vs = j > 0 ? v[c - g.nx] : 0.0;
-  const double vn = j < g.ny - 1 ? v[c + g.nx] : 0.0;
-  const double* Tx = g.Tx + (size_t)j * (g.nx + 1) + i;
-  const double* Ty = g.Ty + (size_t)j * g.nx + i;
-  const double wx = Tx[1] * (vc - ve) - Tx[0] * (vw - vc);
-  const double wy = Ty[g.nx] * (vc - vn) - Ty[0] * (vs - vc);
-  return wx + wy;
-}
-
 __global__ void k_matvec(Geo g, const double* __restrict__ v, double* __restrict__ w) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int j = blockIdx.y;
-  if (i >= g.nx) return;
-  w[(size_t)j * g.nx + i] = apply_A(g, v, i, j);
+  const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
+  if (i < g.nx) w[(size_t)j * g.nx + i] = apply_A(g, v, i, j);
 }
-
-__global__ void k_residual(Geo g, const double* __restrict__ r, const double* __restrict__ z, double* __restrict__ rho) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int j = blockIdx.y;
-  if (i >= g.nx) return;
-  const size_t c = (size_t)j * g.nx + i;
-  rho[c] = r[c] - apply_A(g, z, i, j);
+__global__ void __launch_bounds__(128) k_matvec_march(Geo g, const double* __restrict__ v, double* __restrict__ w, int rows) {
+  const int j0 = blockIdx.y * rows;
+  stencil_march<1>(g, v, stencil_col0(), j0, min(j0 + rows, g.ny), [](size_t) { return 0.0; },
+                   [&](size_t c, double s) { w[c] = s; });
 }
 
 // Face velocities u_f (positive along +axis).
@@ -160,13 +141,10 @@ cudaError_t launch_assemble(const Geo& g, const int* bc_kind, const double* cons
 }
 
 cudaError_t launch_matvec(const Geo& g, const double* v, double* w, cudaStream_t st) {
-  k_matvec<<<row_grid(g.nx, g.ny, 128), 128, 0, st>>>(g, v, w);
-  count_launch(1);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_residual(const Geo& g, const double* r, const double* z, double* rho, cudaStream_t st) {
-  k_residual<<<row_grid(g.nx, g.ny, 128), 128, 0, st>>>(g, r, z, rho);
+  if (stencil_marches(g.nx, g.ny))
+    k_matvec_march<<<stencil_grid(g.nx, g.ny), 128, 0, st>>>(g, v, w, stencil_rows(g.nx, g.ny));
+  else
+    k_matvec<<<row_grid(g.nx, g.ny, 128), 128, 0, st>>>(g, v, w);
   count_launch(1);
   return cudaGetLastError();
 }

@@ -38,16 +38,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_matvec_dot(Geo g, const double*
   const size_t n = (size_t)g.nx * g.ny;
   for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < n; c += (size_t)gridDim.x * blockDim.x) {
     const int i = (int)(c % g.nx), j = (int)(c / g.nx);
-    const double zc = z[c];
-    const double zw = i > 0 ? z[c - 1] : 0.0;
-    const double ze = i < g.nx - 1 ? z[c + 1] : 0.0;
-    const double zs = j > 0 ? z[c - g.nx] : 0.0;
-    const double zn = j < g.ny - 1 ? z[c + g.nx] : 0.0;
-    const double* Tx = g.Tx + (size_t)j * (g.nx + 1) + i;
-    const double* Ty = g.Ty + (size_t)j * g.nx + i;
-    const double wx = Tx[1] * (zc - ze) - Tx[0] * (zw - zc);
-    const double wy = Ty[g.nx] * (zc - zn) - Ty[0] * (zs - zc);
-    const double wc = wx + wy;
+    const double wc = apply_A(g, z, i, j);
     w[c] = wc;
     v[0] += wc * v0[c];
     v[1] += wc * wc;
@@ -137,16 +128,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_residual_norm(Geo g, const doub
   const size_t n = (size_t)g.nx * g.ny;
   for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < n; c += (size_t)gridDim.x * blockDim.x) {
     const int i = (int)(c % g.nx), j = (int)(c / g.nx);
-    const double pc = p[c];
-    const double pw = i > 0 ? p[c - 1] : 0.0;
-    const double pe = i < g.nx - 1 ? p[c + 1] : 0.0;
-    const double ps = j > 0 ? p[c - g.nx] : 0.0;
-    const double pn = j < g.ny - 1 ? p[c + g.nx] : 0.0;
-    const double* Tx = g.Tx + (size_t)j * (g.nx + 1) + i;
-    const double* Ty = g.Ty + (size_t)j * g.nx + i;
-    const double wx = Tx[1] * (pc - pe) - Tx[0] * (pw - pc);
-    const double wy = Ty[g.nx] * (pc - pn) - Ty[0] * (ps - pc);
-    const double rc = b[c] - (wx + wy);
+    const double rc = b[c] - apply_A(g, p, i, j);
     r[c] = rc;
     v[0] += rc * rc;
   }
@@ -350,20 +332,7 @@ __global__ void __launch_bounds__(ARN_THREADS, 1) k_arnoldi_ls(Geo g, LsArgs a) 
       r[e] = 0.0;
       if (c < hi) {
         const int i = (int)(c % g.nx), jj = (int)(c / g.nx);
-        const double* z = a.z;
-        const double zc = z[c];
-        const double zw = i > 0 ? z[c - 1] : 0.0;
-        const double ze = i < g.nx - 1 ? z[c + 1] : 0.0;
-        const double zs = jj > 0 ? z[c - g.nx] : 0.0;
-        const double zn = jj < g.ny - 1 ? z[c + g.nx] : 0.0;
-        const double* Tx = g.Tx + (size_t)jj * (g.nx + 1) + i;
-        const double* Ty = g.Ty + (size_t)jj * g.nx + i;
-        // the four face fluxes from the differences (no cancellation against a diagonal term), one
-        // product and three FMAs
-        double f = Tx[1] * (zc - ze);
-        f = fma(Tx[0], zc - zw, f);
-        f = fma(Ty[g.nx], zc - zn, f);
-        r[e] = fma(Ty[0], zc - zs, f);
+        r[e] = apply_A(g, a.z, i, jj);
       }
     }
 #pragma unroll

@@ -1946,27 +1946,23 @@ cudaError_t launch_basis(const Geo& g, const void* Linv, int LS, bool fp32, cons
 // (z == nullptr: r; else the sweep's residual r - A z in FP64, rounded once), so that each box
 // fetches its cells with one round of asynchronous copies instead of forming them
 __global__ void k_stage32(Geo g, const double* __restrict__ r, const double* __restrict__ z, float* __restrict__ out) {
-  const int gx = blockIdx.x * blockDim.x + threadIdx.x, gy = blockIdx.y;
-  if (gx >= g.nx) return;
-  const size_t c = (size_t)gy * g.nx + gx;
-  double v = r[c];
-  if (z) {
-    const double zc = z[c];
-    const double zw = gx > 0 ? z[c - 1] : 0.0, ze = gx < g.nx - 1 ? z[c + 1] : 0.0;
-    const double zs = gy > 0 ? z[c - g.nx] : 0.0, zn = gy < g.ny - 1 ? z[c + g.nx] : 0.0;
-    const size_t cx = (size_t)gy * (g.nx + 1) + gx;
-    // r minus the four face fluxes, each from its difference: four subtractions and four FMAs
-    v = fma(-g.Tx[cx + 1], zc - ze, v);
-    v = fma(-g.Tx[cx], zc - zw, v);
-    v = fma(-g.Ty[c + g.nx], zc - zn, v);
-    v = fma(-g.Ty[c], zc - zs, v);
-  }
-  out[c] = (float)v;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
+  if (i >= g.nx) return;
+  const size_t c = (size_t)j * g.nx + i;
+  out[c] = (float)(z ? face_sum<-1>(g, z, i, j, r[c]) : r[c]);
+}
+__global__ void __launch_bounds__(128) k_stage32_march(Geo g, const double* __restrict__ r, const double* __restrict__ z,
+                                                     float* __restrict__ out, int rows) {
+  const int j0 = blockIdx.y * rows;
+  stencil_march<-1>(g, z, stencil_col0(), j0, min(j0 + rows, g.ny), [&](size_t c) { return r[c]; },
+                    [&](size_t c, double s) { out[c] = (float)s; });
 }
 
 cudaError_t launch_stage32(const Geo& g, const double* r, const double* z, float* out, cudaStream_t st) {
-  dim3 grid((g.nx + 255) / 256, g.ny);
-  k_stage32<<<grid, 256, 0, st>>>(g, r, z, out);
+  if (z && stencil_marches(g.nx, g.ny))
+    k_stage32_march<<<stencil_grid(g.nx, g.ny), 128, 0, st>>>(g, r, z, out, stencil_rows(g.nx, g.ny));
+  else
+    k_stage32<<<dim3((g.nx + 255) / 256, g.ny), 256, 0, st>>>(g, r, z, out);
   count_launch(1);
   return cudaGetLastError();
 }

@@ -41,16 +41,7 @@ __global__ void __launch_bounds__(mrcm::RED_THREADS) k_residual_norm_static(mrcm
   const size_t n = (size_t)g.nx * g.ny;
   for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < n; c += (size_t)gridDim.x * blockDim.x) {
     const int i = (int)(c % g.nx), j = (int)(c / g.nx);
-    const double pc = p[c];
-    const double pw = i > 0 ? p[c - 1] : 0.0;
-    const double pe = i < g.nx - 1 ? p[c + 1] : 0.0;
-    const double ps = j > 0 ? p[c - g.nx] : 0.0;
-    const double pn = j < g.ny - 1 ? p[c + g.nx] : 0.0;
-    const double* Tx = g.Tx + (size_t)j * (g.nx + 1) + i;
-    const double* Ty = g.Ty + (size_t)j * g.nx + i;
-    const double wx = Tx[1] * (pc - pe) - Tx[0] * (pw - pc);
-    const double wy = Ty[g.nx] * (pc - pn) - Ty[0] * (ps - pc);
-    const double rc = b[c] - (wx + wy);
+    const double rc = b[c] - mrcm::apply_A(g, p, i, j);
     r[c] = rc;
     v[0] += rc * rc;
   }
