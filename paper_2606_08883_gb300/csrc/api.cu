@@ -673,7 +673,6 @@ mrcm_status mrcm_gmres_solve(mrcm_handle h, const double* b, double* p, double* 
   double* bnorm_d = beta_d + 1;
   double* partials = at<double>(h, L.red);
   unsigned* counter = reinterpret_cast<unsigned*>(partials + RED_DOUBLES);
-  unsigned* bar = counter + 1;
   int* flags = at<int>(h, L.flags);
   bool fused = true;  // fused Arnoldi kernel, unless the vector is too long for one co-resident wave
   if (!h->rb) {
@@ -742,7 +741,7 @@ mrcm_status mrcm_gmres_solve(mrcm_handle h, const double* b, double* p, double* 
           cudaError_t ea = cudaErrorNotSupported;
           if (fused)
             ea = launch_arnoldi(g, zj, V, j, n, H, ldh, cs, sn, gv, out, w, at<double>(h, L.apart),
-                                at<double>(h, L.atot), at<double>(h, L.aT), bar, flags, st);
+                                at<double>(h, L.atot), at<double>(h, L.aT), flags, st);
           if (ea == cudaErrorNotSupported) {
             fused = false;
             (void)cudaGetLastError();

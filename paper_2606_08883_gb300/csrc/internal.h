@@ -353,7 +353,7 @@ cudaError_t launch_mf_factor(const MfDev& m, const Plan& P, const double* ab, in
 cudaError_t launch_mf_solve(const MfDev& m, const double* mom0, double* g, int* flags, cudaStream_t st);
 cudaError_t launch_arnoldi(const Geo& g, const double* z, double* V, int j, size_t n, double* H, int ldh, double* cs,
                            double* sn, double* gv, double* out, double* wbuf, double* part, double* tot, double* Tm,
-                           unsigned* bar, int* flags, cudaStream_t st);
+                           int* flags, cudaStream_t st);
 
 // Krylov helpers (k_krylov.cu)
 cudaError_t launch_norm2(const double* x, size_t n, double* partials, unsigned* counter, double* out,

@@ -149,6 +149,14 @@ __global__ void __launch_bounds__(RED_THREADS) k_residual_norm(Geo g, const doub
 // h_i = (T a)_i for i < j is a product instead of a sequential solve, and the last coefficient is
 // the MGS recurrence itself, h_j = a_j - sum_k r_k h_k.
 //
+// Barriers: arrivals add to a counter that only grows (a multiple of the grid's CTAs between launches;
+// zeroed with the flags at each set-up), so a barrier is one release and one acquire poll, and work that
+// only the last block needs (the rotations) runs between its arrival and its wait.  Vectors of up to
+// ARN_CLUSTER_N elements take one cluster of up to eight CTAs and the cluster's hardware barrier instead;
+// with few CTAs every one forms all totals itself and the second barrier goes.  With the finer cut of
+// arn_grid a step takes 34.8 -> 25.4 us at 64^2, 37.7 -> 27.7 at 128^2, 47.4 -> 43.0 at 512^2, 87.3 -> 83.3 at
+// 1024^2 (the FP64 pipe's share of it 1, 2, 18 and 72 us).
+//
 // Per step: one sweep over the basis that forms a_k and r_k together for every k < j (one read of
 // v_k), plus (w, v_j) and ||A z_j||^2; one sweep for w -= V h and ||w||^2; three grid barriers.
 // Each block owns one contiguous slice of the vectors.  GB300's FP64 rate (2 DFMA/clk/SM, 64-clock
@@ -180,7 +188,7 @@ struct LsArgs {
   double* part;         // (2 ldh + 3) x gridDim partial sums
   double* tot;          // 2 ldh + 3 totals
   double* Tm;           // (I + R)^-1, row-major lower, leading dimension ldh
-  unsigned* bar;
+  unsigned long long* bar;
   int* flags;
   int stage_T;          // 1: rows of T staged in shared memory (fits), 0: read from global
 };
@@ -190,6 +198,10 @@ constexpr int DOT_UNROLL = 4;   // elements of the swept basis vector in flight 
 constexpr int UPD_EL = 2;       // vector elements per thread in the update sweep
 constexpr int UPD_UU = 2;       // basis vectors per ring stage
 constexpr int UPD_DS = 3;       // ring stages
+constexpr int ARN_CHUNK = 256;        // fewest elements per CTA
+constexpr int ARN_CLUSTER = 8;        // most CTAs of the one-cluster form
+constexpr int ARN_CLUSTER_N = ARN_CLUSTER * 512;   // elements up to which it is taken
+constexpr int ARN_DIRECT = 32;        // CTAs up to which every CTA forms all totals
 constexpr int ROW_TPR = 4;      // threads per row of T in the coefficient product
 constexpr int ARN_SMALL = 5 * 264;                               // a | r | h | cs | sn (doubles)
 constexpr int ARN_RING = UPD_DS * UPD_UU * UPD_EL * ARN_THREADS;  // doubles
@@ -308,6 +320,54 @@ __device__ __forceinline__ void update_ring(const double* __restrict__ V, size_t
   }
 }
 
+// Barrier over the CTAs of the launch, split into arrival and bounded wait.  CL: one cluster.
+template <bool CL>
+struct ArnBarrier {
+  unsigned long long* count;
+  int* flags;
+  unsigned long long target = 0;   // thread 0: the count that completes the current barrier
+  // thread 0, before its first arrival: fewer than gridDim.x arrivals of the launch can be in the count
+  __device__ __forceinline__ void init() {
+    if (!CL && threadIdx.x == 0) target = *(volatile unsigned long long*)count / gridDim.x * gridDim.x;
+  }
+  __device__ __forceinline__ void arrive() {
+    if (CL) {
+      __syncwarp();
+      asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+      return;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      __threadfence();
+      asm volatile("red.release.gpu.global.add.u64 [%0], 1;" ::"l"(count) : "memory");
+      target += gridDim.x;
+    }
+  }
+  // false if the wait gave up (FLAG_TIMEOUT is set; the caller returns)
+  __device__ __forceinline__ bool wait() {
+    if (CL) {
+      asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+      return true;
+    }
+    __shared__ int s_ok;
+    if (threadIdx.x == 0) {
+      s_ok = 0;
+      for (long long spins = 0; spins < BARRIER_SPIN_LIMIT; ++spins) {
+        unsigned long long c;
+        asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(c) : "l"(count) : "memory");
+        if (c >= target) {
+          s_ok = 1;
+          break;
+        }
+      }
+      if (!s_ok) atomicOr(flags, FLAG_TIMEOUT);
+    }
+    __syncthreads();
+    return s_ok != 0;
+  }
+};
+
+template <bool CL>
 __global__ void __launch_bounds__(ARN_THREADS, 1) k_arnoldi_ls(Geo g, LsArgs a) {
   extern __shared__ double sh[];      // small arrays | ring (update) or staged rows of T
   __shared__ double sm[32];
@@ -321,6 +381,8 @@ __global__ void __launch_bounds__(ARN_THREADS, 1) k_arnoldi_ls(Geo g, LsArgs a) 
   const size_t lo = (size_t)b * chunk < n ? (size_t)b * chunk : n;
   const size_t hi = lo + chunk < n ? lo + chunk : n;
   double* w = a.wbuf;
+  ArnBarrier<CL> bar{a.bar, a.flags};
+  bar.init();
   const double* vj = a.V + (size_t)j * n;
   double* ring = sh + ARN_SMALL;
   // 1. w = A z_j on the slice (4 elements per thread, all loads before the stores)
@@ -401,20 +463,25 @@ __global__ void __launch_bounds__(ARN_THREADS, 1) k_arnoldi_ls(Geo g, LsArgs a) 
       if (lane == 16) s_dot[2 * warp + 1] = v;
     }
     __syncthreads();
-    if (tid < 2 * nr) {
-      const int uu = tid >> 1, which = tid & 1;
+    // the parts' sums, a warp per sum where there are many parts, else a thread
+    for (int x = wpt > 6 ? warp : tid; x < 2 * nr; x += wpt > 6 ? nw : nt) {
+      const int uu = x >> 1, which = x & 1;
       const int t = j - (u0 + uu);
       double acc = 0.0;
-      for (int q = 0; q < wpt; ++q) acc += s_dot[2 * (uu * wpt + q) + which];
+      if (wpt > 6) {
+        acc = warp_sum(lane < wpt ? s_dot[2 * (uu * wpt + lane) + which] : 0.0);
+      } else {
+        for (int q = 0; q < wpt; ++q) acc += s_dot[2 * (uu * wpt + q) + which];
+      }
       const int slot = which == 0 ? t : (t < j ? j + 1 + t : 2 * j + 1);
-      a.part[(size_t)slot * G + b] = acc;
+      if (wpt <= 6 || lane == 0) a.part[(size_t)slot * G + b] = acc;
     }
     __syncthreads();
   }
-  __threadfence();
-  if (!grid_barrier(a.bar, a.flags)) return;
+  bar.arrive();
+  if (!bar.wait()) return;
   // 3. copy rows 1..j-1 of T (lower part, row i at offset i(i-1)/2) to shared memory while the
-  //    totals are formed, one dot per block (in block order)
+  //    totals are formed, one dot per block (in block order), or all of them in every block of a small grid
   const int ldt = a.ldh;
   double* Ts = ring;
   if (a.stage_T) {
@@ -422,28 +489,31 @@ __global__ void __launch_bounds__(ARN_THREADS, 1) k_arnoldi_ls(Geo g, LsArgs a) 
       for (int k = lane; k < i; k += 32) cp_async8(Ts + i * (i - 1) / 2 + k, a.Tm + (size_t)i * ldt + k);
     cp_async_commit();
   }
-  if (warp == 0)
-    for (int t = b; t < nd; t += G) {
+  const bool direct = G <= ARN_DIRECT;
+  if (direct || warp == 0)
+    for (int t = direct ? warp : b; t < nd; t += direct ? nw : G) {
       double acc = 0.0;
       for (int k = lane; k < G; k += 32) acc += *((volatile double*)&a.part[(size_t)t * G + k]);
       acc = warp_sum(acc);
-      if (lane == 0) a.tot[t] = acc;
+      if (lane == 0) (direct ? sh : a.tot)[t] = acc;
     }
-  __threadfence();
-  if (!grid_barrier(a.bar, a.flags)) {
-    cp_async_wait<0>();
-    return;
+  if (!direct) {
+    bar.arrive();
+    if (!bar.wait()) {
+      cp_async_wait<0>();
+      return;
+    }
   }
   // 4. MGS coefficients: h_i = a_i + sum_{k<i} T_ik a_k (i < j, ROW_TPR threads per row), then
   //    h_j = a_j - sum_k r_k h_k; the new row t_jk = -sum_{i=k}^{j-1} r_i T_ik of T is split over
   //    the blocks by column and read from the next step on.
   double* sa = sh;               // a[0..j]
   double* sr = sa + (j + 1);     // r[0..j-1]
-  double* shh = sr + j;          // h[0..j]
+  double* shh = sr + j + 1;      // h[0..j]   (||A z_j||^2 stands between r and h)
   double* scs = shh + (j + 1);   // cs[0..j-1] (last block)
   double* ssn = scs + j;         // sn[0..j-1] (last block)
-  for (int t = tid; t < nd - 1; t += nt) sa[t] = *((volatile double*)&a.tot[t]);
-  const double wn2 = *((volatile double*)&a.tot[nd - 1]);
+  if (!direct)
+    for (int t = tid; t < nd; t += nt) sa[t] = *((volatile double*)&a.tot[t]);
   if (b == G - 1)
     for (int k = tid; k < j; k += nt) {
       scs[k] = a.cs[k];
@@ -451,6 +521,7 @@ __global__ void __launch_bounds__(ARN_THREADS, 1) k_arnoldi_ls(Geo g, LsArgs a) 
     }
   cp_async_wait<0>();
   __syncthreads();
+  const double wn2 = sa[nd - 1];
   for (int rb = warp * (32 / ROW_TPR); rb < j; rb += nw * (32 / ROW_TPR)) {   // rb is warp-uniform
     const int i = rb + lane / ROW_TPR, q = lane % ROW_TPR;
     double acc = 0.0;
@@ -485,11 +556,6 @@ __global__ void __launch_bounds__(ARN_THREADS, 1) k_arnoldi_ls(Geo g, LsArgs a) 
     if (lane == 0) shh[j] = sa[j] - acc;
   }
   __syncthreads();
-  // previous rotations on column j: last block, warp 0, before its share of the update
-  if (b == G - 1 && warp == 0) {
-    const double x = givens_scan(scs, ssn, shh, a.H + (size_t)j * a.ldh, j, lane);
-    if (lane == 0) s_x = x;
-  }
   // 5. w -= V h on the slice, ||w||^2 (UPD_EL elements per thread; warp-uniform counts except
   //    in the one warp that holds the slice end)
   double nrm = 0.0;
@@ -509,8 +575,14 @@ __global__ void __launch_bounds__(ARN_THREADS, 1) k_arnoldi_ls(Geo g, LsArgs a) 
   }
   nrm = block_sum(nrm, sm);
   if (tid == 0) a.part[(size_t)nd * G + b] = nrm;
-  __threadfence();
-  if (!grid_barrier(a.bar, a.flags)) return;
+  bar.arrive();
+  // previous rotations on column j: the last block's warp 1, between its arrival and the wait
+  if (b == G - 1 && warp == 1) {
+    const double x = givens_scan(scs, ssn, shh, a.H + (size_t)j * a.ldh, j, lane);
+    if (lane == 0) s_x = x;
+  }
+  __syncwarp();
+  if (!bar.wait()) return;
   // 6. h_{j+1,j} = ||w||, v_{j+1} = w / h_{j+1,j}; last rotation of the column (last block)
   if (warp == 0) {
     double acc = 0.0;
@@ -558,32 +630,77 @@ __global__ void __launch_bounds__(ARN_THREADS, 1) k_arnoldi_ls(Geo g, LsArgs a) 
   }
 }
 
+// CTAs for a vector of n elements: the FP64 pipe takes (3 j + 13) n operations per step, so vectors that
+// would leave SMs idle are cut finer than a thread per element (256^2 on 64 CTAs of 1,024 elements: 38.6 us
+// a step, on every SM: 29.4)
+static int arn_grid(int sms, size_t n) {
+  return (int)std::max<size_t>(1, std::min<size_t>((size_t)sms, (n + ARN_CHUNK - 1) / ARN_CHUNK));
+}
+
 // Returns cudaErrorNotSupported when one co-resident wave cannot cover the grid.
 cudaError_t launch_arnoldi(const Geo& g, const double* z, double* V, int j, size_t n, double* H, int ldh, double* cs,
                            double* sn, double* gv, double* out, double* wbuf, double* part, double* tot, double* Tm,
-                           unsigned* bar, int* flags, cudaStream_t st) {
+                           int* flags, cudaStream_t st) {
   struct Occ {
-    int sms = 0, per_sm = 0;
+    int sms = 0, per_sm = 0, clusters = 0;
   };
   static const Occ occ = [] {  // thread-safe one-time initialisation (request workers call this)
     Occ o;
     int dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&o.sms, cudaDevAttrMultiProcessorCount, dev);
-    raise_smem_limit<k_arnoldi_ls>();
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o.per_sm, k_arnoldi_ls, ARN_THREADS, ARN_SMEM_MAX);
+    raise_smem_limit<k_arnoldi_ls<false>>();
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o.per_sm, k_arnoldi_ls<false>, ARN_THREADS, ARN_SMEM_MAX);
+    if (raise_smem_limit<k_arnoldi_ls<true>>() == cudaSuccess) {
+      cudaLaunchConfig_t cfg = {};
+      cudaLaunchAttribute at[1];
+      at[0].id = cudaLaunchAttributeClusterDimension;
+      at[0].val.clusterDim.x = ARN_CLUSTER;
+      at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+      cfg.gridDim = dim3(ARN_CLUSTER);
+      cfg.blockDim = dim3(ARN_THREADS);
+      cfg.dynamicSmemBytes = ARN_SMEM_MAX;
+      cfg.attrs = at;
+      cfg.numAttrs = 1;
+      if (cudaOccupancyMaxActiveClusters(&o.clusters, k_arnoldi_ls<true>, &cfg) != cudaSuccess) o.clusters = 0;
+    }
+    (void)cudaGetLastError();
     return o;
   }();
   const int sms = occ.sms, per_sm = occ.per_sm;
-  int grid = (int)std::min<size_t>((size_t)sms, (n + ARN_THREADS - 1) / ARN_THREADS);
-  if (grid < 1) grid = 1;
+  int grid = arn_grid(sms, n);
+  const bool cluster = n <= (size_t)ARN_CLUSTER_N && occ.clusters > 0;
+  if (cluster)
+    for (int p = ARN_CLUSTER; p > 0; p >>= 1)   // the largest power of two up to the CTAs that have elements
+      if (grid >= p) {
+        grid = p;
+        break;
+      }
   if (grid > ARNOLDI_MAX_BLOCKS || per_sm < 1 || ldh > 257) return cudaErrorNotSupported;
   const size_t tri = (size_t)j * (j > 0 ? j - 1 : 0) / 2;
   const int stage_T = 8 * (ARN_SMALL + std::max<size_t>(ARN_RING, tri)) <= (size_t)ARN_SMEM_MAX ? 1 : 0;
   const size_t smem = 8 * (ARN_SMALL + (stage_T ? std::max<size_t>(ARN_RING, tri) : (size_t)ARN_RING));
-  LsArgs a{z, V, j, n, H, ldh, cs, sn, gv, out, wbuf, part, tot, Tm, bar, flags, stage_T};
-  void* args[] = {(void*)&g, (void*)&a};
-  cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_arnoldi_ls, dim3(grid), dim3(ARN_THREADS), args, smem, st);
+  // the barrier's arrivals share the flag block, which each set-up zeroes (words 32, 33)
+  LsArgs a{z, V, j, n, H, ldh, cs, sn, gv, out, wbuf, part, tot, Tm,
+           reinterpret_cast<unsigned long long*>(flags + 32), flags, stage_T};
+  cudaError_t e;
+  if (cluster) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = grid;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(ARN_THREADS);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    e = cudaLaunchKernelEx(&cfg, k_arnoldi_ls<true>, g, a);
+  } else {
+    void* args[] = {(void*)&g, (void*)&a};
+    e = cudaLaunchCooperativeKernel((const void*)k_arnoldi_ls<false>, dim3(grid), dim3(ARN_THREADS), args, smem, st);
+  }
   if (e == cudaSuccess) count_launch(1);
   return e;
 }
@@ -688,8 +805,7 @@ cudaError_t launch_update(double* p, const double* Z, size_t n, const double* H,
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  int grid = (int)std::min<size_t>((size_t)sms, (n + ARN_THREADS - 1) / ARN_THREADS);
-  if (grid < 1) grid = 1;
+  const int grid = arn_grid(sms, n);
   k_update_p<<<grid, ARN_THREADS, sizeof(double) * (ARN_SMALL + ARN_RING), st>>>(p, Z, n, ybuf, k);
   count_launch(1);
   return cudaGetLastError();
