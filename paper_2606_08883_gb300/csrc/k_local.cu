@@ -589,23 +589,12 @@ __global__ void __launch_bounds__(64) k_factor_sweep(Geo g, int kind, int LS, fl
 // 26, and both lose to it from 256 boxes on).  At most 128 registers are taken up to 40 columns: with
 // four boxes per SM the pipe is 84 % busy, and a wider launch ends in a shorter last wave.  Against
 // one-CTA Cholesky, L^-1 and L^-T L^-1 in shared memory (164 block barriers per line): set-up of
-// 512^2 cells in 40-wide boxes 5.5 -> 3.8 ms, of 1024^2 in 36-wide boxes 17.8 -> 10.0 ms, of 64^2 in
+// 512^2 cells in 40-wide boxes 5.5 -> 3.7 ms, of 1024^2 in 36-wide boxes 17.8 -> 9.8 ms, of 64^2 in
 // 20-wide boxes 0.70 -> 0.48 ms.  Errors against 80-bit solves are 0.8 to 1.0 times those of the
 // Cholesky route (log-normal, channel and white-noise boxes).
 // --------------------------------------------------------------------------------------------
 constexpr int FR_HT = 64;
 
-// 1 / d from the hardware's reciprocal estimate (about 20 bits) by one cubic step,
-// r <- r + r (e + e^2) with e = 1 - d r: three dependent FMAs (within 2.3e-16 of 1 / d).  A result
-// outside the normal range takes the division.
-__device__ __forceinline__ double recip(double d) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
-  const double e = fma(-d, r, 1.0);
-  const double v = fma(r, fma(e, e, e), r);
-  const int ex = __double2hiint(v) & 0x7ff00000;   // integer tests: FP64 compares would take the FP64 pipe
-  return ex != 0 && ex != 0x7ff00000 ? v : 1.0 / d;
-}
 // d > 0 and finite, by its bits
 __device__ __forceinline__ bool positive_finite(double d) {
   const long long v = __double_as_longlong(d);
@@ -627,7 +616,7 @@ __global__ void __launch_bounds__(2 * FR_HT, WMAX <= 40 ? 4 : 1)
     double c[2][WMAX + 1];   // pivot column, double-buffered; slot WMAX belongs to the unused entries
     double w[WMAX + 1];      // the same divided by the pivot
     double d[WMAX + 1], o[WMAX + 1], e[WMAX + 1];   // the line's diagonal, right and previous-line couplings
-    double r;                // 1 / pivot
+    double nr;               // -1 / pivot (negated once: an FP64 negation is an FP64 instruction)
   };
   __shared__ Half sm_all[2];
   __shared__ double s_mid[NP];    // the bottom recursion's last S^-1, for the middle line
@@ -708,15 +697,15 @@ __global__ void __launch_bounds__(2 * FR_HT, WMAX <= 40 ? 4 : 1)
 #pragma unroll
         for (int i0 = 0; i0 < WMAX; i0 += 32)
           if (i0 + lane < w) sm.w[i0 + lane] = c[i0 + lane] * ri;
-        if (lane == 0) sm.r = ri;
+        if (lane == 0) sm.nr = -ri;
       }
       half_sync(half);
-      const double ri = sm.r;
+      const double nri = sm.nr;
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         const int i = ij[r] >> 8, j = ij[r] & 255;
         double v = fma(-sm.w[i], c[j], a[r]);
-        if (i == k || j == k) v = i == j ? -ri : sm.w[i == k ? j : i];
+        if (i == k || j == k) v = i == j ? nri : sm.w[i == k ? j : i];
         a[r] = v;
         if (i == k + 1 || j == k + 1) cn[i == k + 1 ? j : i] = v;
       }
