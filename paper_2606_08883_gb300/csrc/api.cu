@@ -175,7 +175,6 @@ MfDev mfdev(mrcm_handle h) {
   m.order = at<int>(h, L.mf_ord);
   m.idx = at<int>(h, L.mf_idx);
   m.asmv = at<int2>(h, L.mf_asm);
-  m.map = at<int>(h, L.mf_map);
   m.task = at<int4>(h, L.mf_task);
   m.F = at<double>(h, L.mf_F);
   m.V = at<double>(h, L.mf_V);
@@ -386,7 +385,6 @@ mrcm_status mrcm_setup(const mrcm_problem* problem, const mrcm_params* params, v
     up(L.mf_ord, HP.mf_order.data(), 4 * HP.mf_order.size());
     up(L.mf_idx, HP.mf_idx.data(), 4 * HP.mf_idx.size());
     up(L.mf_asm, HP.mf_asm.data(), 4 * HP.mf_asm.size());
-    up(L.mf_map, HP.mf_map.data(), 4 * HP.mf_map.size());
     up(L.mf_task, HP.mf_task.data(), 4 * HP.mf_task.size());
     up(L.mf_item, HP.mf_item.data(), sizeof(MfItem) * HP.mf_item.size());
     up(L.mf_inv, HP.mf_inv.data(), 4 * HP.mf_inv.size());

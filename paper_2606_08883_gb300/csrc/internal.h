@@ -20,7 +20,7 @@ namespace mrcm {
 // interfaces on the separator of its rectangle of subdomains, or every interface inside a leaf
 // rectangle) and the update unknowns U (the interfaces on the rectangle's boundary), P first.  The
 // dense front F = [F11 F12; F21 F22] (row-major, f = np + nu) is overwritten by F11^-1,
-// D = F11^-1 F12 and S = F22 - F21 D; B = F21 F11^-1 (nu x np) follows F.
+// D = F11^-1 F12 and S = F22 - F21 D; B = F21 F11^-1 (nu x np) and a copy of F12 (np x nu) follow F.
 struct MfFront {
   long long fo;   // offset (doubles) of F in the front buffer
   int np, nu;
@@ -29,7 +29,6 @@ struct MfFront {
   int ao, na;     // its assembly pairs
   int nch;        // children (0..2)
   int ch[2];      // child front ids
-  int mo[2];      // offsets of the children's maps
   int par;        // parent front id (-1 at the root)
 };
 // One part of a front in the solve: forward rows [u0, u1) of B, backward rows [p0, p1) of [F11^-1 D];
@@ -39,7 +38,7 @@ struct MfItem {
 };
 constexpr int MF_LEAF = 16;       // leaf rectangles of at most this many subdomains
 constexpr int MF_MAX_NP = 128;    // largest pivot block (its inverse is formed in shared memory)
-constexpr int MF_TILE = 32;       // tile of the D, B and S products
+constexpr int MF_TILE = 16;       // tile of the D, B and S products
 constexpr int MF_PARTS = 304;     // parts per level that the solve aims at (two CTAs on each of 152 SMs)
 constexpr int MF_PART_ROWS = 8;   // rows below which a part is not split further
 constexpr int MF_STAGE = 6144;    // doubles of front rows that a part stages in shared memory
@@ -74,7 +73,6 @@ struct Plan {
   std::vector<int> mf_level;       // [levels + 1] starts of the levels in mf_order
   std::vector<int> mf_idx;         // unknowns of each front, P then U
   std::vector<int> mf_asm;         // (dst, src) pairs: front-local offset, band offset of G
-  std::vector<int> mf_map;         // child U position -> parent front position
   std::vector<int> mf_task;        // (front, kind, r0, c0) tile tasks
   std::vector<int> mf_task_b;      // [levels + 1] starts of each level's D / B tasks
   std::vector<int> mf_task_c;      // [levels + 1] starts of each level's Schur-complement tasks
@@ -111,7 +109,7 @@ struct Layout {
   size_t gtr;                             // Robin coefficients of the Gamma faces, k_local.cu
   size_t rto, rtl;                        // t_R of the Robin box faces of the oversampled / subdomain boxes
   size_t gbML, gbMU, gbX, gbY, gbF, gbC;  // blocked substitution (above COARSE_DENSE_MAX), k_coarse.cu
-  size_t mf_fr, mf_ord, mf_idx, mf_asm, mf_map, mf_task;   // multifrontal tables, k_mf.cu
+  size_t mf_fr, mf_ord, mf_idx, mf_asm, mf_task;   // multifrontal tables, k_mf.cu
   size_t mf_item, mf_inv, mf_rhs;         // its solve's work list, message slots and right-hand sides
   size_t mf_F, mf_V, mf_scr, mf_msg;      // fronts, solve vectors, scratch words, messages (upward, then x)
   size_t rho, zt;                         // FP32 staged right-hand sides (k_stage32), apply output scratch
@@ -328,7 +326,6 @@ struct MfDev {
   const int* order;
   const int* idx;
   const int2* asmv;
-  const int* map;
   const int4* task;
   const MfItem* item;   // [nitem] the solve's parts, level by level
   const int2* inv;      // message slots of each front position's children (-1: none)

@@ -13,6 +13,8 @@
 // then backward, x_P = F11^-1 v_P - D x_U.  Every product has a fixed order, so the solution is
 // deterministic.  A zero or non-finite pivot, or |S| above NOPIV_MAX_GROWTH max |G|, sets
 // FLAG_NOPIV_REJECTED and the caller falls back to the pivoted band LU of k_coarse.cu.
+#include <algorithm>
+
 #include <cooperative_groups.h>
 
 #include "common.cuh"
@@ -23,78 +25,154 @@ constexpr int MF_THREADS = 256;
 constexpr int MF_GJ_CL = 8;          // CTAs of the cluster that inverts a large pivot block
 constexpr int MF_GJ_CLUSTER_NP = 64; // pivot blocks this large (and divisible by MF_GJ_CL) use it
 
-// largest of a non-negative double across the CTA into an 8-byte maximum in global memory (the
-// bit patterns of non-negative doubles order like the values; +inf above every finite value)
-__device__ __forceinline__ void cta_max_to(double v, unsigned long long* dst) {
-  __shared__ double red[MF_THREADS / 32];
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  __syncthreads();
-  if (lane == 0) red[wid] = v;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double m = red[0];
-    for (int i = 1; i < (int)(blockDim.x >> 5); ++i) m = fmax(m, red[i]);
-    atomicMax(dst, (unsigned long long)__double_as_longlong(m));
+// Magnitudes as bit patterns (those of non-negative doubles order like the values; anything not finite counts
+// as +inf), compared as integers: FP64 compares, like FP64 negations, take the FP64 pipe.
+__device__ __forceinline__ unsigned long long mag(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffULL;
+  return b < 0x7ff0000000000000ULL ? b : 0x7ff0000000000000ULL;
+}
+__device__ __forceinline__ bool nonzero_finite(double d) {
+  const unsigned long long b = mag(d);
+  return b != 0 && b != 0x7ff0000000000000ULL;
+}
+// the largest magnitude across the CTA into a maximum in global memory
+__device__ __forceinline__ void cta_max_to(unsigned long long v, unsigned long long* dst) {
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long u = __shfl_xor_sync(0xffffffffu, v, o);
+    v = u > v ? u : v;
   }
+  if ((threadIdx.x & 31) == 0 && v) atomicMax(dst, v);
 }
 
-__device__ __forceinline__ double mag(double v) { return isfinite(v) ? fabs(v) : __longlong_as_double(0x7ff0000000000000LL); }
-
-// C (M x N) = (acc ? C : 0) + alpha A (M x K) B (K x N), row-major operands with leading
-// dimensions, in global or shared memory; one CTA of MF_THREADS, 32 x 32 output tiles with 2 x 2
-// outputs per thread, K in chunks of 32 staged in shared memory (sm: 2048 doubles).  Returns the
-// largest |C| written (+inf for a non-finite entry).
-__device__ double cta_gemm(int M, int N, int K, const double* A, int lda, const double* B, int ldb, double* C,
-                           int ldc, double alpha, bool acc, double* sm) {
-  double* As = sm;          // As[k * 32 + r] = A[m0 + r][k0 + k]
-  double* Bs = sm + 1024;   // Bs[k * 32 + c] = B[k0 + k][n0 + c]
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  double cmax = 0.0;
-  for (int m0 = 0; m0 < M; m0 += 32)
-    for (int n0 = 0; n0 < N; n0 += 32) {
-      double c00 = 0.0, c01 = 0.0, c10 = 0.0, c11 = 0.0;
-      for (int k0 = 0; k0 < K; k0 += 32) {
-        for (int t = tid; t < 1024; t += MF_THREADS) {
-          const int k = t >> 5, r = t & 31;
-          As[t] = (m0 + r < M && k0 + k < K) ? A[(size_t)(m0 + r) * lda + k0 + k] : 0.0;
-          Bs[t] = (k0 + k < K && n0 + r < N) ? B[(size_t)(k0 + k) * ldb + n0 + r] : 0.0;
-        }
-        __syncthreads();
-#pragma unroll 8
-        for (int k = 0; k < 32; ++k) {
-          const double a0 = As[k * 32 + ty], a1 = As[k * 32 + ty + 16];
-          const double b0 = Bs[k * 32 + tx], b1 = Bs[k * 32 + tx + 16];
-          c00 = fma(a0, b0, c00);
-          c01 = fma(a0, b1, c01);
-          c10 = fma(a1, b0, c10);
-          c11 = fma(a1, b1, c11);
-        }
-        __syncthreads();
-      }
-      const double cv[2][2] = {{c00, c01}, {c10, c11}};
-#pragma unroll
-      for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          const int r = m0 + ty + 16 * i, c = n0 + tx + 16 * j;
-          if (r < M && c < N) {
-            double* p = C + (size_t)r * ldc + c;
-            const double v = (acc ? *p : 0.0) + alpha * cv[i][j];
-            *p = v;
-            cmax = fmax(cmax, mag(v));
-          }
-        }
-    }
-  return cmax;
+// One MF_TILE x MF_TILE tile of C (rows x cols of it) = (acc ? C : 0) + alpha A (rows x K) B (K x cols),
+// row-major operands with leading dimensions in global memory, one output per thread of the CTA; both
+// operands are staged in shared memory (sm: MF_TILE (2 K + 1) + K doubles).  Returns the magnitude of the
+// entry written.
+__device__ unsigned long long cta_tile(int rows, int cols, int K, const double* A, int lda, const double* B, int ldb, double* C, int ldc,
+                           double alpha, bool acc, double* sm) {
+  double* As = sm;                            // [MF_TILE][K + 1]
+  double* Bs = sm + MF_TILE * (K + 1);        // [K][MF_TILE]
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  for (int r = wid; r < MF_TILE; r += MF_THREADS / 32)
+    for (int k = lane; k < K; k += 32) As[r * (K + 1) + k] = r < rows ? A[(size_t)r * lda + k] : 0.0;
+  for (int t = tid; t < K * MF_TILE; t += MF_THREADS) {
+    const int k = t / MF_TILE, c = t % MF_TILE;
+    Bs[t] = c < cols ? B[(size_t)k * ldb + c] : 0.0;
+  }
+  const int r = tid / MF_TILE, c = tid % MF_TILE;
+  const bool on = r < rows && c < cols;
+  const double old = on && acc ? C[(size_t)r * ldc + c] : 0.0;
+  __syncthreads();
+  double s0 = 0.0, s1 = 0.0;
+  int k = 0;
+  for (; k + 1 < K; k += 2) {
+    s0 = fma(As[r * (K + 1) + k], Bs[k * MF_TILE + c], s0);
+    s1 = fma(As[r * (K + 1) + k + 1], Bs[(k + 1) * MF_TILE + c], s1);
+  }
+  if (k < K) s0 = fma(As[r * (K + 1) + k], Bs[k * MF_TILE + c], s0);
+  const double v = fma(alpha, s0 + s1, old);
+  if (on) C[(size_t)r * ldc + c] = v;
+  return on ? mag(v) : 0ULL;
 }
 
 __device__ __forceinline__ unsigned long long* mf_stats(const MfDev& m) {
   return reinterpret_cast<unsigned long long*>(m.scr + 2);
 }
 
-// One CTA per front of a level: assembly (zero, the original entries of the pivot rows and
-// columns, the children's Schur complements in child order) and F11^-1 in place.
+// Gauss-Jordan inversion in registers of np rows by nc columns [c0, c0 + nc) of the pivot block (entry
+// t = thread + MF_THREADS r of the nc-wide rows; pivot k takes w_i = a_ik / a_kk and the row a_k., then a_ij -= w_i a_kj
+// off row and column k, row k = a_kj / a_kk, column k = -w_i, a_kk = 1 / a_kk).  The column is published by the
+// step before, over the whole block, the row by this CTA.  Bound by the FP64 pipe of its SM: an update is one FMA
+// per entry with every lane busy, the reciprocal and the scaled column cost a handful per warp, and the column is
+// kept negated because an FP64 negation per entry is an FP64 instruction too (with that and a division a pivot of
+// a 48-wide block took 2.0 us; now 1.6).
+template <int R>
+struct GjBlock {
+  double a[R];
+  int ij[R];   // row << 8 | column; unused entries: the spare slot (np, nc)
+  int nr;      // rounds with entries
+  __device__ __forceinline__ void load(const double* F, int f, int np, int nc) {
+    const int di = MF_THREADS / nc, dj = MF_THREADS - di * nc;
+    int i = threadIdx.x / nc, j = threadIdx.x - i * nc;
+    nr = (np * nc + MF_THREADS - 1) / MF_THREADS;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const bool on = i < np;
+      ij[r] = on ? i << 8 | j : np << 8 | nc;
+      a[r] = on ? F[(size_t)i * f + j] : 0.0;
+      i += di;
+      j += dj;
+      if (j >= nc) {
+        j -= nc;
+        ++i;
+      }
+    }
+  }
+  __device__ __forceinline__ void store(double* F, int f, int np) const {
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+      if ((ij[r] >> 8) < np) F[(size_t)(ij[r] >> 8) * f + (ij[r] & 255)] = a[r];
+  }
+  // row and column k (own column kc, or none if outside) into the published arrays
+  __device__ __forceinline__ void publish(int k, int kc, double* row, double* col) const {
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int i = ij[r] >> 8, j = ij[r] & 255;
+      if (i == k) row[j] = a[r];
+      if (j == kc) col[i] = a[r];
+    }
+  }
+  // pivot k with nw (the scaled column, negated), row k, row k times rp (1 / pivot); publishes row and column k + 1
+  __device__ __forceinline__ void pivot(int k, int kc, const double* nw, const double* row, const double* rowr, double rp,
+                                        double* next_row, double* next_col) {
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      if (r >= nr) break;
+      const int i = ij[r] >> 8, j = ij[r] & 255;
+      const double ci = nw[i];
+      double v = fma(ci, row[j], a[r]);
+      if (i == k) v = j == kc ? rp : rowr[j];
+      else if (j == kc) v = ci;
+      a[r] = v;
+      if (i == k + 1) next_row[j] = v;
+      if (j == kc + 1) next_col[i] = v;
+    }
+  }
+};
+
+// The children's Schur complements into the fronts of a level, a row of F per warp: entry (i, j) is the sum over
+// the children that hold both unknowns (their message slots say which and where), 0 elsewhere.  With one CTA per
+// front adding its children entry by entry, the upper levels' assembly alone took 25 to 45 us each.
+__global__ void __launch_bounds__(MF_THREADS) k_mf_gather(MfDev m, int first) {
+  const MfFront fr = m.fr[m.order[first + blockIdx.x]];
+  const int f = fr.np + fr.nu, i = blockIdx.y * (MF_THREADS / 32) + (threadIdx.x >> 5);
+  if (i >= f) return;
+  const int2 si = m.inv[fr.io + i];
+  const double* S[2] = {nullptr, nullptr};   // row of the child's S that belongs to row i
+  int wo[2] = {0, 0};
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    const int slot = c == 0 ? si.x : si.y;
+    if (c < fr.nch && slot >= 0) {
+      const MfFront cf = m.fr[fr.ch[c]];
+      const int fc = cf.np + cf.nu;
+      wo[c] = cf.wo;
+      S[c] = m.F + cf.fo + (size_t)(cf.np + slot - cf.wo) * fc + cf.np;
+    }
+  }
+  double* row = m.F + fr.fo + (size_t)i * f;
+#pragma unroll 4
+  for (int j = threadIdx.x & 31; j < f; j += 32) {
+    const int2 sj = m.inv[fr.io + j];
+    double v = S[0] && sj.x >= 0 ? S[0][sj.x - wo[0]] : 0.0;
+    if (S[1] && sj.y >= 0) v += S[1][sj.y - wo[1]];
+    row[j] = v;
+  }
+}
+
+// One CTA per front of a level: the original entries of the pivot rows and columns, and F11^-1 of the blocks that
+// one CTA inverts.
+template <int R>
 __global__ void __launch_bounds__(MF_THREADS) k_mf_front(MfDev m, const double* __restrict__ ab, int first,
                                                          int* flags) {
   extern __shared__ __align__(16) double smd[];
@@ -102,15 +180,13 @@ __global__ void __launch_bounds__(MF_THREADS) k_mf_front(MfDev m, const double* 
   const MfFront fr = m.fr[fid];
   const int np = fr.np, nu = fr.nu, f = np + nu;
   double* __restrict__ F = m.F + fr.fo;
-  for (size_t t = threadIdx.x; t < (size_t)f * f; t += MF_THREADS) F[t] = 0.0;
-  __syncthreads();
-  // assembly in batches of AB entries per thread, every load of a batch issued before its stores
-  // (the positions within one batch, and within one child, are distinct)
+  // the original entries on top of the children's (k_mf_gather), in batches of AB per thread, every load of a batch
+  // issued before its stores (the positions are distinct)
   constexpr int AB = 8;
-  double amax = 0.0;
+  unsigned long long amax = 0;
   for (int t0 = threadIdx.x; t0 < fr.na; t0 += AB * MF_THREADS) {
     int dst[AB];
-    double v[AB];
+    double v[AB], o[AB];
 #pragma unroll
     for (int e = 0; e < AB; ++e) {
       const int t = t0 + e * MF_THREADS;
@@ -123,88 +199,62 @@ __global__ void __launch_bounds__(MF_THREADS) k_mf_front(MfDev m, const double* 
       }
     }
 #pragma unroll
+    for (int e = 0; e < AB; ++e) o[e] = dst[e] >= 0 ? F[dst[e]] : 0.0;
+#pragma unroll
     for (int e = 0; e < AB; ++e)
       if (dst[e] >= 0) {
-        F[dst[e]] = v[e];
-        amax = fmax(amax, mag(v[e]));
+        F[dst[e]] = o[e] + v[e];
+        const unsigned long long b = mag(v[e]);
+        amax = b > amax ? b : amax;
       }
-  }
-  __syncthreads();
-  for (int c = 0; c < fr.nch; ++c) {
-    const MfFront cf = m.fr[c == 0 ? fr.ch[0] : fr.ch[1]];
-    const int fc = cf.np + cf.nu, nuc = cf.nu;
-    const double* __restrict__ S = m.F + cf.fo + (size_t)cf.np * fc + cf.np;
-    const int* mp = m.map + (c == 0 ? fr.mo[0] : fr.mo[1]);
-    for (int t0 = threadIdx.x; t0 < nuc * nuc; t0 += AB * MF_THREADS) {
-      size_t dst[AB];
-      double v[AB], o[AB];
-#pragma unroll
-      for (int e = 0; e < AB; ++e) {
-        const int t = t0 + e * MF_THREADS;
-        dst[e] = ~(size_t)0;
-        v[e] = o[e] = 0.0;
-        if (t < nuc * nuc) {
-          const int i = t / nuc, j = t - i * nuc;
-          dst[e] = (size_t)mp[i] * f + mp[j];
-          v[e] = S[(size_t)i * fc + j];
-        }
-      }
-#pragma unroll
-      for (int e = 0; e < AB; ++e)
-        if (dst[e] != ~(size_t)0) o[e] = F[dst[e]];
-#pragma unroll
-      for (int e = 0; e < AB; ++e)
-        if (dst[e] != ~(size_t)0) F[dst[e]] = o[e] + v[e];
-    }
-    __syncthreads();
   }
   cta_max_to(amax, mf_stats(m));
+  __syncthreads();
+  // F12 aside: the tiles of D = F11^-1 F12 overwrite it while others still read it
+  double* Fc = F + (size_t)f * f + (size_t)nu * np;
+  for (int i = threadIdx.x >> 5; i < np; i += MF_THREADS / 32)
+    for (int j = threadIdx.x & 31; j < nu; j += 32) Fc[(size_t)i * nu + j] = F[(size_t)i * f + np + j];
   if (np >= MF_GJ_CLUSTER_NP && np % MF_GJ_CL == 0) return;   // F11^-1 by k_mf_gj_cluster
-  // Gauss-Jordan on F11 (np x np) in shared memory: pivot k takes the scaled row r_k = A_k. / a_kk
-  // and the column c_k = A_.k, then a_ij -= c_i r_j off row and column k, row k = r_k, column
-  // k = -c_k / a_kk, a_kk = 1 / a_kk; after the np pivots A = F11^-1
-  double* A = smd;
-  double* rk = A + np * np;
-  double* ck = rk + np;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int i = wid; i < np; i += MF_THREADS / 32)
-    for (int j = lane; j < np; j += 32) A[i * np + j] = F[(size_t)i * f + j];
+  // F11^-1 (at most R MF_THREADS entries: the launcher picks R by the level's largest block)
+  const int tid = threadIdx.x;
+  double* row = smd;                      // [2][np + 1] row k, double-buffered
+  double* col = row + 2 * (np + 1);       // [2][np + 1] column k
+  double* w = col + 2 * (np + 1);         // [np + 1] column k / pivot, negated
+  double* rowr = w + np + 1;              // [np + 1] row k / pivot
+  double* s_r = rowr + np + 1;            // 1 / pivot
+  for (int t = tid; t < 6 * (np + 1); t += MF_THREADS) smd[t] = 0.0;
+  GjBlock<R> blk;
+  blk.load(F, f, np, np);
+  __syncthreads();
+  blk.publish(0, 0, row, col);
   __syncthreads();
   bool bad = false;
   for (int k = 0; k < np; ++k) {
-    double d = A[k * np + k];
-    if (!(fabs(d) > 0.0) || !isfinite(d)) {
-      bad = true;
-      d = 1.0;
-    }
-    const double r = 1.0 / d;
-    for (int j = threadIdx.x; j < np; j += MF_THREADS) {
-      rk[j] = A[k * np + j] * r;
-      ck[j] = A[j * np + k];
+    const int c = (k & 1) * (np + 1), n = np + 1 - c;
+    if (tid < np) {
+      double d = col[c + k];
+      if (!nonzero_finite(d)) {
+        bad = true;
+        d = 1.0;
+      }
+      const double r = recip(d);
+      w[tid] = col[c + tid] * -r;
+      rowr[tid] = row[c + tid] * r;
+      if (tid == 0) *s_r = r;
     }
     __syncthreads();
-    for (int i = wid; i < np; i += MF_THREADS / 32) {
-      const double ci = ck[i];
-      for (int j = lane; j < np; j += 32) {
-        double v;
-        if (i == k) v = j == k ? r : rk[j];
-        else if (j == k) v = -ci * r;
-        else v = fma(-ci, rk[j], A[i * np + j]);
-        A[i * np + j] = v;
-      }
-    }
+    blk.pivot(k, k, w, row + c, rowr, *s_r, row + n, col + n);
     __syncthreads();
   }
-  for (int i = wid; i < np; i += MF_THREADS / 32)
-    for (int j = lane; j < np; j += 32) F[(size_t)i * f + j] = A[i * np + j];
-  if (bad && lane == 0) atomicOr(flags, FLAG_NOPIV_REJECTED);
+  blk.store(F, f, np);
+  if (bad) atomicOr(flags, FLAG_NOPIV_REJECTED);
 }
 
 // F11^-1 of a large pivot block by the same Gauss-Jordan steps, over a cluster of MF_GJ_CL CTAs:
-// CTA q keeps columns [q cw, (q + 1) cw) of F11 in shared memory (cw = np / MF_GJ_CL); per pivot the
-// owner of column k publishes it (double-buffered), one cluster barrier, every CTA copies it through
-// distributed shared memory and updates its columns.  Entry by entry the arithmetic is that of the
-// one-CTA form.  One cluster per front of the level; fronts too small for it return at once.
+// CTA q keeps columns [q cw, (q + 1) cw) of F11 in its registers (cw = np / MF_GJ_CL); per pivot the
+// owner of column k has published it (double-buffered), one cluster barrier, every CTA reads it through
+// distributed shared memory, scales it and updates its columns.  Entry by entry the arithmetic is that of
+// the one-CTA form.  One cluster per front of the level; fronts too small for it return at once.
 __global__ void __launch_bounds__(MF_THREADS, 1) k_mf_gj_cluster(MfDev m, int first, int* flags) {
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
@@ -216,79 +266,67 @@ __global__ void __launch_bounds__(MF_THREADS, 1) k_mf_gj_cluster(MfDev m, int fi
   if (np < MF_GJ_CLUSTER_NP || np % MF_GJ_CL != 0) return;   // uniform over the cluster
   const int cw = np / MF_GJ_CL, c0 = q * cw;
   double* F = m.F + fr.fo;
-  double* A = smd;                 // [np][cw] this CTA's columns
-  double* pub = A + np * cw;       // [2][np] the pivot column, published by its owner
-  double* col = pub + 2 * np;      // [np] the pivot column, copied
-  double* rk = col + np;           // [cw] this CTA's part of the scaled pivot row
+  constexpr int R = MF_MAX_NP * MF_MAX_NP / MF_GJ_CL / MF_THREADS;
+  double* pub = smd;                   // [2][np + 1] the pivot column, published by its owner
+  double* w = pub + 2 * (np + 1);      // [np + 1] the same divided by the pivot, negated
+  double* row = w + np + 1;            // [2][cw + 1] this CTA's part of the pivot row
+  double* rowr = row + 2 * (cw + 1);   // [cw + 1] the same divided by the pivot
+  double* s_r = rowr + cw + 1;         // 1 / pivot
   const int tid = threadIdx.x;
-  for (int t = tid; t < np * cw; t += MF_THREADS) {
-    const int i = t / cw, jj = t - i * cw;
-    A[t] = F[(size_t)i * f + c0 + jj];
-  }
+  for (int t = tid; t < 3 * (np + 1) + 3 * (cw + 1); t += MF_THREADS) smd[t] = 0.0;
+  GjBlock<R> blk;
+  blk.load(F + c0, f, np, cw);
   __syncthreads();
+  blk.publish(0, q == 0 ? 0 : -1, row, pub);
   bool bad = false;
   for (int k = 0; k < np; ++k) {
-    const int owner = k / cw, kk = k - owner * cw;
-    double* pb = pub + (k & 1) * np;
-    if (q == owner)
-      for (int i = tid; i < np; i += MF_THREADS) pb[i] = A[i * cw + kk];
+    const int owner = k / cw, kc = k - c0;   // this CTA's column of pivot k, in [0, cw) at its owner only
+    const int c = k & 1, n = c ^ 1;
     cl.sync();
-    const double* rp = cl.map_shared_rank(pb, owner);
-    for (int i = tid; i < np; i += MF_THREADS) col[i] = rp[i];
-    __syncthreads();
-    double d = col[k];
-    if (!(fabs(d) > 0.0) || !isfinite(d)) {
-      bad = true;
-      d = 1.0;
-    }
-    const double r = 1.0 / d;
-    for (int jj = tid; jj < cw; jj += MF_THREADS) rk[jj] = A[k * cw + jj] * r;
-    __syncthreads();
-    for (int t = tid; t < np * cw; t += MF_THREADS) {
-      const int i = t / cw, jj = t - i * cw;
-      const int j = c0 + jj;
-      double v;
-      if (i == k) v = j == k ? r : rk[jj];
-      else if (j == k) v = -col[i] * r;
-      else v = fma(-col[i], rk[jj], A[t]);
-      A[t] = v;
+    const double* rp = cl.map_shared_rank(pub + c * (np + 1), owner);
+    if (tid < np) {   // np <= MF_MAX_NP < MF_THREADS
+      double d = rp[k];
+      const double ci = rp[tid];
+      if (!nonzero_finite(d)) {
+        bad = true;
+        d = 1.0;
+      }
+      const double r = recip(d);
+      w[tid] = ci * -r;
+      if (tid < cw) rowr[tid] = row[c * (cw + 1) + tid] * r;
+      if (tid == 0) *s_r = r;
     }
     __syncthreads();
+    blk.pivot(k, kc, w, row + c * (cw + 1), rowr, *s_r, row + n * (cw + 1), pub + n * (np + 1));
   }
   cl.sync();   // no CTA leaves while another may still read its published column
-  for (int t = tid; t < np * cw; t += MF_THREADS) {
-    const int i = t / cw, jj = t - i * cw;
-    F[(size_t)i * f + c0 + jj] = A[t];
-  }
-  if (bad && tid == 0) atomicOr(flags, FLAG_NOPIV_REJECTED);
+  blk.store(F + c0, f, np);
+  if (bad) atomicOr(flags, FLAG_NOPIV_REJECTED);
 }
 
-// Tile tasks of a level: kind 0, columns c0.. of D = F11^-1 F12 (in place of F12, from a shared
-// copy); kind 1, rows r0.. of B = F21 F11^-1; kind 2, the (r0, c0) tile of S = F22 - F21 D.
+// Tile tasks of a level, MF_TILE x MF_TILE outputs at (r0, c0) each: kind 0, of D = F11^-1 F12 (in place of
+// F12, from its copy); kind 1, of B = F21 F11^-1; kind 2, of S = F22 - F21 D.  The fronts are few and small, so
+// the tiles are too: a 32-wide slab of a leaf's D (48 pivots) kept one SM's FP64 pipe 42 us while most SMs had
+// none; now 13 us for the level (16 leaves), 138 -> 71 us for 256.
 __global__ void __launch_bounds__(MF_THREADS) k_mf_tiles(MfDev m, int first) {
+  static_assert(MF_TILE * MF_TILE == MF_THREADS, "one output per thread");
   extern __shared__ __align__(16) double smd[];
   const int4 tk = m.task[first + blockIdx.x];
   const MfFront fr = m.fr[tk.x];
-  const int np = fr.np, nu = fr.nu, f = np + nu;
+  const int np = fr.np, nu = fr.nu, f = np + nu, r0 = tk.z, c0 = tk.w;
   double* F = m.F + fr.fo;
   double* Bx = F + (size_t)f * f;
-  double* stage = smd + 2048;
+  const double* Fc = Bx + (size_t)nu * np;
   if (tk.y == 0) {
-    const int cols = min(MF_TILE, nu - tk.w);
-    for (int t = threadIdx.x; t < np * MF_TILE; t += MF_THREADS) {
-      const int i = t / MF_TILE, j = t - i * MF_TILE;
-      stage[t] = j < cols ? F[(size_t)i * f + np + tk.w + j] : 0.0;
-    }
-    __syncthreads();
-    cta_gemm(np, cols, np, F, f, stage, MF_TILE, F + np + tk.w, f, 1.0, false, smd);
+    cta_tile(min(MF_TILE, np - r0), min(MF_TILE, nu - c0), np, F + (size_t)r0 * f, f, Fc + c0, nu,
+             F + (size_t)r0 * f + np + c0, f, 1.0, false, smd);
   } else if (tk.y == 1) {
-    const int rows = min(MF_TILE, nu - tk.z);
-    cta_gemm(rows, np, np, F + (size_t)(np + tk.z) * f, f, F, f, Bx + (size_t)tk.z * np, np, 1.0, false, smd);
+    cta_tile(min(MF_TILE, nu - r0), min(MF_TILE, np - c0), np, F + (size_t)(np + r0) * f, f, F + c0, f,
+             Bx + (size_t)r0 * np + c0, np, 1.0, false, smd);
   } else {
-    const int rows = min(MF_TILE, nu - tk.z), cols = min(MF_TILE, nu - tk.w);
-    const double smax = cta_gemm(rows, cols, np, F + (size_t)(np + tk.z) * f, f, F + np + tk.w, f,
-                                 F + (size_t)(np + tk.z) * f + np + tk.w, f, -1.0, true, smd);
-    cta_max_to(smax, mf_stats(m) + 1);
+    const unsigned long long s = cta_tile(min(MF_TILE, nu - r0), min(MF_TILE, nu - c0), np, F + (size_t)(np + r0) * f, f, F + np + c0, f,
+                              F + (size_t)(np + r0) * f + np + c0, f, -1.0, true, smd);
+    cta_max_to(s, mf_stats(m) + 1);
   }
 }
 
@@ -299,29 +337,45 @@ __global__ void k_mf_check(MfDev m, int* flags) {
 }
 
 cudaError_t launch_mf_factor(const MfDev& m, const Plan& P, const double* ab, int* flags, cudaStream_t st) {
-  const size_t sm_front = 8 * ((size_t)P.mf_max_np * P.mf_max_np + 2 * (size_t)P.mf_max_np);
-  const size_t sm_tiles = 8 * (2048 + (size_t)P.mf_max_np * MF_TILE);
   // the limits go to the device maximum once (raise_smem_limit): request workers launch these kernels
   // from several host threads with different sizes, and a per-launch limit could be lowered by
   // another thread between its set and its launch
-  cudaError_t e = raise_smem_limit<k_mf_front>();
-  if (e == cudaSuccess) e = raise_smem_limit<k_mf_tiles>();
+  cudaError_t e = raise_smem_limit<k_mf_tiles>();
   if (e != cudaSuccess) return e;
   e = cudaMemsetAsync(m.scr + 2, 0, 16, st);   // the statistics; the solve epoch runs on
   if (e != cudaSuccess) return e;
   for (int L = 0; L + 1 < (int)P.mf_level.size(); ++L) {
     const int nf = P.mf_level[L + 1] - P.mf_level[L];
+    // shared memory by the level's own pivot blocks, so that several small fronts share an SM
+    bool big = false;                   // a pivot block for the cluster form
+    size_t np_one = 1, np_max = 1;      // the largest block of the one-CTA form, and of all
+    int f_max = 1;
+    for (int i = P.mf_level[L]; i < P.mf_level[L + 1]; ++i) {
+      const MfFront& fr = P.mf_front[P.mf_order[i]];
+      const bool cl = fr.np >= MF_GJ_CLUSTER_NP && fr.np % MF_GJ_CL == 0;
+      big = big || cl;
+      if (!cl) np_one = std::max(np_one, (size_t)fr.np);
+      np_max = std::max(np_max, (size_t)fr.np);
+      f_max = std::max(f_max, fr.np + fr.nu);
+    }
+    const size_t sm_tiles = 8 * (MF_TILE * (2 * np_max + 1) + np_max);
     if (nf > 0) {
-      k_mf_front<<<nf, MF_THREADS, sm_front, st>>>(m, ab, P.mf_level[L], flags);
+      k_mf_gather<<<dim3(nf, (f_max + MF_THREADS / 32 - 1) / (MF_THREADS / 32)), MF_THREADS, 0, st>>>(m, P.mf_level[L]);
       count_launch(1);
-      bool big = false;   // a pivot block for the cluster form
-      for (int i = P.mf_level[L]; i < P.mf_level[L + 1]; ++i) {
-        const MfFront& fr = P.mf_front[P.mf_order[i]];
-        big = big || (fr.np >= MF_GJ_CLUSTER_NP && fr.np % MF_GJ_CL == 0);
-      }
+      const int rounds = (int)((np_one * np_one + MF_THREADS - 1) / MF_THREADS);
+      const size_t sm = 8 * (6 * (np_one + 1) + 1);
+#define MRCM_MF_FRONT(R) k_mf_front<R><<<nf, MF_THREADS, sm, st>>>(m, ab, P.mf_level[L], flags)
+      if (rounds <= 2) MRCM_MF_FRONT(2);
+      else if (rounds <= 4) MRCM_MF_FRONT(4);
+      else if (rounds <= 9) MRCM_MF_FRONT(9);
+      else if (rounds <= 16) MRCM_MF_FRONT(16);
+      else if (rounds <= 25) MRCM_MF_FRONT(25);
+      else if (rounds <= 36) MRCM_MF_FRONT(36);
+      else MRCM_MF_FRONT(64);
+#undef MRCM_MF_FRONT
+      count_launch(1);
       if (big) {
-        const size_t sm_gj = 8 * ((size_t)P.mf_max_np * (P.mf_max_np / MF_GJ_CL) + 3 * (size_t)P.mf_max_np +
-                                  P.mf_max_np / MF_GJ_CL);
+        const size_t sm_gj = 8 * (3 * (np_max + 1) + 3 * (np_max / MF_GJ_CL + 1) + 1);
         cudaError_t e2 = raise_smem_limit<k_mf_gj_cluster>();
         if (e2 != cudaSuccess) return e2;
         cudaLaunchConfig_t cfg = {};

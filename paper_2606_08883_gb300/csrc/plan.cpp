@@ -141,7 +141,6 @@ std::string make_plan(const mrcm_problem& p, const mrcm_params& q, Plan& P) {
     P.mf_front.clear();
     P.mf_idx.clear();
     P.mf_asm.clear();
-    P.mf_map.clear();
     P.mf_task.clear();
     P.mf_item.clear();
     P.mf_inv.clear();
@@ -248,7 +247,6 @@ static bool plan_mf(Plan& P) {
   }
   std::vector<int> pos(P.NC, -1);
   P.mf_asm.clear();
-  P.mf_map.clear();
   size_t fo = 0;
   int wo = 0;
   P.mf_max_np = P.mf_max_f = 0;
@@ -268,17 +266,15 @@ static bool plan_mf(Plan& P) {
     fr.na = (int)P.mf_asm.size() / 2 - fr.ao;
     for (int c = 0; c < fr.nch; ++c) {
       const MfFront& cf = P.mf_front[fr.ch[c]];
-      fr.mo[c] = (int)P.mf_map.size();
       for (int t = 0; t < cf.nu; ++t) {
         const int p = pos[P.mf_idx[cf.io + cf.np + t]];
         if (p < 0) return false;
-        P.mf_map.push_back(p);
         P.mf_inv[2 * (size_t)(fr.io + p) + c] = cf.wo + t;
       }
     }
     for (int t = 0; t < fs; ++t) pos[P.mf_idx[fr.io + t]] = -1;
     fr.fo = (long long)fo;
-    fo += (size_t)fs * fs + (size_t)fr.nu * fr.np;
+    fo += (size_t)fs * fs + 2 * (size_t)fr.nu * fr.np;
     fr.wo = wo;
     wo += fr.nu;
     P.mf_max_np = std::max(P.mf_max_np, fr.np);
@@ -302,10 +298,11 @@ static bool plan_mf(Plan& P) {
     for (int i = P.mf_level[L]; i < (int)P.mf_order.size(); ++i) {
       const int f = P.mf_order[i];
       const MfFront& fr = P.mf_front[f];
-      for (int t = 0; t < fr.nu; t += MF_TILE) {
-        P.mf_task.insert(P.mf_task.end(), {f, 0, 0, t});   // D columns t ..
-        P.mf_task.insert(P.mf_task.end(), {f, 1, t, 0});   // B rows t ..
-      }
+      for (int t = 0; t < fr.nu; t += MF_TILE)
+        for (int k = 0; k < fr.np; k += MF_TILE) {
+          P.mf_task.insert(P.mf_task.end(), {f, 0, k, t});   // D rows k .., columns t ..
+          P.mf_task.insert(P.mf_task.end(), {f, 1, t, k});   // B rows t .., columns k ..
+        }
     }
     P.mf_task_c[L] = (int)P.mf_task.size() / 4;
     for (int i = P.mf_level[L]; i < (int)P.mf_order.size(); ++i) {
@@ -474,7 +471,6 @@ Layout make_layout(const Plan& P, const mrcm_params& q) {
   L.mf_ord = take(4 * P.mf_order.size());
   L.mf_idx = take(4 * P.mf_idx.size());
   L.mf_asm = take(4 * P.mf_asm.size());
-  L.mf_map = take(4 * P.mf_map.size());
   L.mf_task = take(4 * P.mf_task.size());
   L.mf_F = take(8 * P.mf_fbuf);
   L.mf_item = take(sizeof(MfItem) * P.mf_item.size());
