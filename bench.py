@@ -378,8 +378,8 @@ NCU_TRAFFIC = {
 # The Arnoldi step's traffic grows with the inner step j: (bytes, j) of the captured launch, scaled
 # to the solve's average launch by the model's algorithmic bytes (krylov_model), in which the basis
 # sweeps that make the traffic grow in proportion.
-NCU_TRAFFIC_KRYLOV = (576.713984e6 + 62.34112e6, 5, "paper_2606_08883_gb300/csrc/k_krylov.cu",
-                      "97bf265e4b30d16c4335a8ef6753b412892351f7adbec2e54e23ce2f20898f0f")
+NCU_TRAFFIC_KRYLOV = (575.922176e6 + 62.312192e6, 5, "paper_2606_08883_gb300/csrc/k_krylov.cu",
+                      "dd5284ab7c281df05a6cb953d85e8180eda17bd8887e149c07abc381ce45ea7b")
 
 
 def krylov_traffic(n, iterations, restart):
