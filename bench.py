@@ -378,8 +378,8 @@ NCU_TRAFFIC = {
 # The Arnoldi step's traffic grows with the inner step j: (bytes, j) of the captured launch, scaled
 # to the solve's average launch by the model's algorithmic bytes (krylov_model), in which the basis
 # sweeps that make the traffic grow in proportion.
-NCU_TRAFFIC_KRYLOV = (575.922176e6 + 62.312192e6, 5, "paper_2606_08883_gb300/csrc/k_krylov.cu",
-                      "dd5284ab7c281df05a6cb953d85e8180eda17bd8887e149c07abc381ce45ea7b")
+NCU_TRAFFIC_KRYLOV = (576.339968e6 + 62.4448e6, 5, "paper_2606_08883_gb300/csrc/k_krylov.cu",
+                      "3621efcce9df04e1d32efe245a1936f6023331f078e795b1fc83a4f8182da5be")
 
 
 def krylov_traffic(n, iterations, restart):

@@ -225,8 +225,6 @@ __global__ void k_check_positive(const double* K, size_t n, int* flags) {
   }
 }
 
-__global__ void k_set(double* p, double v) { *p = v; }
-
 void bc_ptrs(mrcm_handle h, const double* ptrs[4]) {
   const size_t len = std::max(h->n[0], h->n[1]);
   const double* bcv = at<double>(h, h->lay.bcv);
@@ -674,7 +672,7 @@ mrcm_status mrcm_gmres_solve(mrcm_handle h, const double* b, double* p, double* 
   int* flags = at<int>(h, L.flags);
   bool fused = true;  // fused Arnoldi kernel, unless the vector is too long for one co-resident wave
   if (!h->rb) {
-    CK(h, cudaHostAlloc(reinterpret_cast<void**>(&h->rb), 2 * sizeof(mrcm_ctx::StepReadback), cudaHostAllocDefault));
+    CK(h, cudaHostAlloc(reinterpret_cast<void**>(&h->rb), 2 * sizeof(StepReport), cudaHostAllocMapped | cudaHostAllocPortable));
     for (cudaEvent_t& e : h->rb_ev) CK(h, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
   }
   std::vector<double> hist;
@@ -684,10 +682,12 @@ mrcm_status mrcm_gmres_solve(mrcm_handle h, const double* b, double* p, double* 
   result->latency_ms = 0.0;
   result->queue_ms = 0.0;
   double hb[2] = {0, 0};
+  // both norms before the first look at either (beta_d and bnorm_d are neighbours)
   CK(h, launch_norm2(bb, n, partials, counter, bnorm_d, st));
-  CK(h, cudaMemcpyAsync(hb, bnorm_d, 8, cudaMemcpyDeviceToHost, st));
+  CK(h, launch_residual_norm(g, bb, p, V, partials, counter, beta_d, st));
+  CK(h, cudaMemcpyAsync(hb, beta_d, 16, cudaMemcpyDeviceToHost, st));
   CK(h, cudaStreamSynchronize(st));
-  const double bnorm = hb[0];
+  const double bnorm = hb[1];
   result->bnorm = bnorm;
   const bool rel = h->prm.tol_relative != 0;
   if (rel && bnorm == 0.0) {
@@ -703,10 +703,7 @@ mrcm_status mrcm_gmres_solve(mrcm_handle h, const double* b, double* p, double* 
     return MRCM_OK;
   }
   const double tol_abs = rel ? h->prm.tol * bnorm : h->prm.tol;
-  CK(h, launch_residual_norm(g, bb, p, V, partials, counter, beta_d, st));
-  double beta = 0.0;
-  CK(h, cudaMemcpyAsync(&beta, beta_d, 8, cudaMemcpyDeviceToHost, st));
-  CK(h, cudaStreamSynchronize(st));
+  double beta = hb[0];
   hist.push_back(beta);
   int it = 0;
   mrcm_status status = MRCM_OK;
@@ -716,10 +713,7 @@ mrcm_status mrcm_gmres_solve(mrcm_handle h, const double* b, double* p, double* 
       status = MRCM_ERR_NOT_CONVERGED;
       break;
     }
-    CK(h, launch_scale(V, beta_d, n, V, st));
-    CK(h, cudaMemsetAsync(gv, 0, 8 * (m + 1), st));
-    k_set<<<1, 1, 0, st>>>(gv, beta);
-    CK(h, cudaGetLastError());
+    CK(h, launch_cycle_start(V, beta_d, n, gv, m, st));
     // Steps are pipelined by one: step j+1 is enqueued before the host reads step j's residual
     // estimate, so the device never waits for the host.  When step j ends the cycle, the extra step
     // has only written V_{j+2}, Z_{j+1}, column j+1 of H, rotation j+1 and g_{j+1..j+2}, none of
@@ -734,11 +728,13 @@ mrcm_status mrcm_gmres_solve(mrcm_handle h, const double* b, double* p, double* 
         mrcm_status rc = apply_T(h, vj, zj, st);
         if (rc != MRCM_OK) return rc;
         double* col = H + (size_t)j * ldh;
+        StepReport* slot = h->rb + (j & 1);   // step j - 2's, read already
+        slot->flags = STEP_PENDING;
         {
           Phase ph(h, MRCM_PH_KRYLOV, st);
           cudaError_t ea = cudaErrorNotSupported;
           if (fused)
-            ea = launch_arnoldi(g, zj, V, j, n, H, ldh, cs, sn, gv, out, w, at<double>(h, L.apart),
+            ea = launch_arnoldi(g, zj, V, j, n, H, ldh, cs, sn, gv, slot, w, at<double>(h, L.apart),
                                 at<double>(h, L.atot), at<double>(h, L.aT), flags, st);
           if (ea == cudaErrorNotSupported) {
             fused = false;
@@ -757,19 +753,23 @@ mrcm_status mrcm_gmres_solve(mrcm_handle h, const double* b, double* p, double* 
             CK(h, ea);
           }
         }
-        mrcm_ctx::StepReadback* slot = h->rb + (j & 1);
-        CK(h, cudaMemcpyAsync(slot->out, out, 24, cudaMemcpyDeviceToHost, st));
-        CK(h, cudaMemcpyAsync(&slot->flags, flags, sizeof(int), cudaMemcpyDeviceToHost, st));
+        if (!fused) {
+          CK(h, cudaMemcpyAsync(slot->out, out, 24, cudaMemcpyDeviceToHost, st));
+          CK(h, cudaMemcpyAsync(&slot->flags, flags, sizeof(int), cudaMemcpyDeviceToHost, st));
+        }
         CK(h, cudaEventRecord(h->rb_ev[j & 1], st));
       }
       if (pend >= 0) {
         CK(h, cudaEventSynchronize(h->rb_ev[pend & 1]));
-        const mrcm_ctx::StepReadback* slot = h->rb + (pend & 1);
+        const StepReport* slot = h->rb + (pend & 1);
         const double ho[3] = {slot->out[0], slot->out[1], slot->out[2]};
         ++it;
-        if (slot->flags & FLAG_TIMEOUT)
+        if (slot->flags == STEP_PENDING || (slot->flags & FLAG_TIMEOUT)) {
+          cudaStreamSynchronize(st);   // the step in flight writes the other slot
           return fail(h, MRCM_ERR_TIMEOUT, "a bounded device wait gave up (Arnoldi grid barrier or local-solve line copy)");
+        }
         if (h->cancel && *h->cancel) {
+          cudaStreamSynchronize(st);
           result->iterations = it;
           return fail(h, MRCM_ERR_CANCELLED, "cancelled");
         }

@@ -179,6 +179,15 @@ constexpr int GBB_NB = 512;              // above it: substitution steps per blo
 enum : int { FLAG_SINGULAR_LOCAL = 1, FLAG_SINGULAR_COARSE = 2, FLAG_NONFINITE = 4, FLAG_TIMEOUT = 8,
              FLAG_NOPIV_REJECTED = 16 };   // the no-pivot coupling LU met a zero pivot or large growth
 
+// What a GMRES step reports to the host, in pinned memory that the step's last kernel writes itself (or a copy,
+// on the unfused path); flags is preset to STEP_PENDING, so a step whose kernel gave up is told apart.
+struct StepReport {
+  double out[4];   // |g_{j+1}|, h_{j+1,j}, ||A z_j||
+  int flags;       // the device status word
+  int pad;
+};
+constexpr int STEP_PENDING = -1;
+
 }  // namespace mrcm
 
 // The handle.
@@ -214,14 +223,9 @@ struct mrcm_ctx {
   size_t ev_used = 0;          // pairs recorded since the last read
   double ph_ms[MRCM_PHASES] = {0};
   long long ph_launch[MRCM_PHASES] = {0};
-  // GMRES step read-back: pinned slots so that step j's residual estimate is read while step j+1
-  // runs (created on the first solve)
-  struct StepReadback {
-    double out[4];
-    int flags;
-    int pad;
-  };
-  StepReadback* rb = nullptr;
+  // two pinned slots, so that step j's residual estimate is read while step j+1 runs (created on the
+  // first solve)
+  mrcm::StepReport* rb = nullptr;
   cudaEvent_t rb_ev[2] = {nullptr, nullptr};
   // second stream for set-up work that overlaps (the Schwarz factors), with its fork / join events
   cudaStream_t side = nullptr;
@@ -349,12 +353,14 @@ cudaError_t launch_mf_factor(const MfDev& m, const Plan& P, const double* ab, in
 // backward down them, every part of a front polling the entries that it needs; the solution goes to g.
 cudaError_t launch_mf_solve(const MfDev& m, const double* mom0, double* g, int* flags, cudaStream_t st);
 cudaError_t launch_arnoldi(const Geo& g, const double* z, double* V, int j, size_t n, double* H, int ldh, double* cs,
-                           double* sn, double* gv, double* out, double* wbuf, double* part, double* tot, double* Tm,
+                           double* sn, double* gv, StepReport* report, double* wbuf, double* part, double* tot, double* Tm,
                            int* flags, cudaStream_t st);
 
 // Krylov helpers (k_krylov.cu)
 cudaError_t launch_norm2(const double* x, size_t n, double* partials, unsigned* counter, double* out,
                          cudaStream_t st);
+// v /= *beta in place, g = (*beta, 0, ..., 0) of m + 1 entries
+cudaError_t launch_cycle_start(double* v, const double* beta, size_t n, double* gv, int m, cudaStream_t st);
 cudaError_t launch_scale(const double* x, const double* denom, size_t n, double* y, cudaStream_t st);
 cudaError_t launch_matvec_dot(const Geo& g, const double* z, const double* v0, double* w, double* partials,
                               unsigned* counter, double* out2, cudaStream_t st);

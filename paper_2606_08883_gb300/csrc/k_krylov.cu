@@ -21,6 +21,15 @@ __global__ void __launch_bounds__(RED_THREADS) k_norm2(const double* __restrict_
   grid_reduce<1>(v, partials, counter, outs, sm, 1);
 }
 
+// Start of a cycle: v_0 = r / beta, g = (beta, 0, ..., 0)
+__global__ void k_cycle_start(double* __restrict__ v, const double* __restrict__ beta, size_t n, double* __restrict__ gv,
+                              int m) {
+  const double d = *beta, r = 1.0 / d;
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) v[i] *= r;
+  if (blockIdx.x == 0)
+    for (int i = threadIdx.x; i <= m; i += blockDim.x) gv[i] = i == 0 ? d : 0.0;
+}
+
 __global__ void k_scale(const double* __restrict__ x, const double* __restrict__ denom, size_t n, double* __restrict__ y) {
   const double d = *denom;
   const double r = d != 0.0 ? 1.0 / d : 0.0;
@@ -183,7 +192,7 @@ struct LsArgs {
   double* cs;
   double* sn;
   double* gv;
-  double* out;          // [0] |g_{j+1}|, [1] h_{j+1,j}, [2] ||A z_j||
+  volatile StepReport* report;   // pinned host memory: |g_{j+1}|, h_{j+1,j}, ||A z_j||, the status word
   double* wbuf;         // w (n)
   double* part;         // (2 ldh + 3) x gridDim partial sums
   double* tot;          // 2 ldh + 3 totals
@@ -612,10 +621,12 @@ __global__ void __launch_bounds__(ARN_THREADS, 1) k_arnoldi_ls(Geo g, LsArgs a) 
     const double gj = a.gv[j];
     a.gv[j + 1] = -s * gj;
     a.gv[j] = c * gj;
-    a.out[0] = fabs(-s * gj);
-    a.out[1] = hn;
-    a.out[2] = sqrt(wn2);
-    a.out[3] = 0.0;
+    // straight to the host's slot: as copies queued behind the kernel, the two read-backs held up the next
+    // application's first kernel
+    a.report->out[0] = fabs(-s * gj);
+    a.report->out[1] = hn;
+    a.report->out[2] = sqrt(wn2);
+    a.report->flags = *(volatile int*)a.flags;
   }
   const double rh = hn != 0.0 ? 1.0 / hn : 0.0;
   double* vn = a.V + (size_t)(j + 1) * n;
@@ -639,7 +650,7 @@ static int arn_grid(int sms, size_t n) {
 
 // Returns cudaErrorNotSupported when one co-resident wave cannot cover the grid.
 cudaError_t launch_arnoldi(const Geo& g, const double* z, double* V, int j, size_t n, double* H, int ldh, double* cs,
-                           double* sn, double* gv, double* out, double* wbuf, double* part, double* tot, double* Tm,
+                           double* sn, double* gv, StepReport* report, double* wbuf, double* part, double* tot, double* Tm,
                            int* flags, cudaStream_t st) {
   struct Occ {
     int sms = 0, per_sm = 0, clusters = 0;
@@ -681,7 +692,7 @@ cudaError_t launch_arnoldi(const Geo& g, const double* z, double* V, int j, size
   const int stage_T = 8 * (ARN_SMALL + std::max<size_t>(ARN_RING, tri)) <= (size_t)ARN_SMEM_MAX ? 1 : 0;
   const size_t smem = 8 * (ARN_SMALL + (stage_T ? std::max<size_t>(ARN_RING, tri) : (size_t)ARN_RING));
   // the barrier's arrivals share the flag block, which each set-up zeroes (words 32, 33)
-  LsArgs a{z, V, j, n, H, ldh, cs, sn, gv, out, wbuf, part, tot, Tm,
+  LsArgs a{z, V, j, n, H, ldh, cs, sn, gv, report, wbuf, part, tot, Tm,
            reinterpret_cast<unsigned long long*>(flags + 32), flags, stage_T};
   cudaError_t e;
   if (cluster) {
@@ -712,6 +723,12 @@ static int red_grid(size_t n) {
 
 cudaError_t launch_norm2(const double* x, size_t n, double* partials, unsigned* counter, double* out, cudaStream_t st) {
   k_norm2<<<red_grid(n), RED_THREADS, 0, st>>>(x, n, partials, counter, out);
+  count_launch(1);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_cycle_start(double* v, const double* beta, size_t n, double* gv, int m, cudaStream_t st) {
+  k_cycle_start<<<red_grid(n), RED_THREADS, 0, st>>>(v, beta, n, gv, m);
   count_launch(1);
   return cudaGetLastError();
 }
