@@ -8,7 +8,7 @@
 //   bottom  S_{h-1} = D_{h-1},  S_J = D_J - E_{J+1} S_{J+1}^-1 E_{J+1}    J = h-2 .. m+1
 //   middle  S_m = D_m - E_m S_{m-1}^-1 E_m - E_{m+1} S_{m+1}^-1 E_{m+1}
 // and only the inverses S_J^-1 are stored (symmetric, packed lower triangle, one line block per
-// line; each by Cholesky S_J = L L^T, L^-1, S_J^-1 = L^-T L^-1), followed by the couplings E_J.  A solve eliminates from both ends
+// line; by a symmetric Gauss-Jordan sweep, in FP32 boxes wider than 36 by Cholesky), followed by the couplings E_J.  A solve eliminates from both ends
 //   u_J = b_J + E_J S_{J-1}^-1 u_{J-1} (top),  u_J = b_J + E_{J+1} S_{J+1}^-1 u_{J+1} (bottom),
 //   x_m = S_m^-1 u_m with u_m = b_m + E_m S_{m-1}^-1 u_{m-1} + E_{m+1} S_{m+1}^-1 u_{m+1},
 // and substitutes back outwards: x_J = S_J^-1 (u_J + E_{J+1} x_{J+1}) above the middle,
