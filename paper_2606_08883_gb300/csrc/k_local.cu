@@ -587,7 +587,7 @@ __global__ void __launch_bounds__(64) k_factor_sweep(Geo g, int kind, int LS, fl
 // pivot: npk / 64 rounded up, all lanes busy, plus the reciprocal (three) and the scaling on one
 // warp (36 wide: 13.5 on average; a 128-thread half needs 8.25 on twice the warps, a one-warp half
 // 26, and both lose to it from 256 boxes on).  At most 128 registers are taken up to 40 columns: with
-// four boxes per SM the pipe is 84 % busy, and a wider launch ends in a shorter last wave.  Against
+// four boxes per SM the pipe is 88 % busy, and a wider launch ends in a shorter last wave.  Against
 // one-CTA Cholesky, L^-1 and L^-T L^-1 in shared memory (164 block barriers per line): set-up of
 // 512^2 cells in 40-wide boxes 5.5 -> 3.7 ms, of 1024^2 in 36-wide boxes 17.8 -> 9.8 ms, of 64^2 in
 // 20-wide boxes 0.70 -> 0.48 ms.  Errors against 80-bit solves are 0.8 to 1.0 times those of the
