@@ -8,7 +8,8 @@
 //   bottom  S_{h-1} = D_{h-1},  S_J = D_J - E_{J+1} S_{J+1}^-1 E_{J+1}    J = h-2 .. m+1
 //   middle  S_m = D_m - E_m S_{m-1}^-1 E_m - E_{m+1} S_{m+1}^-1 E_{m+1}
 // and only the inverses S_J^-1 are stored (symmetric, packed lower triangle, one line block per
-// line; by a symmetric Gauss-Jordan sweep, in FP32 boxes wider than 36 by Cholesky), followed by the couplings E_J.  A solve eliminates from both ends
+// line; FP64 and FP32 boxes wider than 36 by Cholesky, L^-1 and L^-T L^-1, narrower FP32 boxes by a symmetric
+// Gauss-Jordan sweep), followed by the couplings E_J.  A solve eliminates from both ends
 //   u_J = b_J + E_J S_{J-1}^-1 u_{J-1} (top),  u_J = b_J + E_{J+1} S_{J+1}^-1 u_{J+1} (bottom),
 //   x_m = S_m^-1 u_m with u_m = b_m + E_m S_{m-1}^-1 u_{m-1} + E_{m+1} S_{m+1}^-1 u_{m+1},
 // and substitutes back outwards: x_J = S_J^-1 (u_J + E_{J+1} x_{J+1}) above the middle,
@@ -577,21 +578,27 @@ __global__ void __launch_bounds__(64) k_factor_sweep(Geo g, int kind, int LS, fl
 // FP64 factorisation, register-resident: one half of the CTA (FR_HT threads) per recursion of the
 // twisted order, the packed lower triangle of the line block spread over the half's registers
 // (entry t = thread + FR_HT r, so a line is written out coalesced).  Each line: the Schur complement
-// from the previous line's inverse, still in the registers, then w pivots of the symmetric
-// Gauss-Jordan sweep (pivot k: w_i = a_ik / a_kk; a_ij -= w_i a_kj off row and column k, which take
-// w, and a_kk = -1 / a_kk), after which the registers hold -S_J^-1.  A pivot publishes its column
-// and then its scaled column through shared memory, two barriers of the half.
+// from the previous line's inverse, still in the registers, then S^-1 = L^-T L^-1 from S = L L^T in
+// place and in one sweep (Bientinesi, Gunter and van de Geijn, 2008).  Before pivot k the rows i >= k
+// hold the Schur complement right of column k and L^-1's work rows left of it, the rows i < k the sum
+// of L^-T L^-1 so far.  With x = column k below the pivot and row k left of it, times 1 / L_kk, and
+// x_k = 1 / L_kk, every entry takes one FMA: a_ij -= x_i x_j in the rows below k, a_ij += x_i x_j in
+// the others, row and column k starting from 0.  Entry by entry these are the operations of a Cholesky
+// factorisation, an inversion of L and the product L^-T L^-1, each summed in increasing k.  The order is
+// part of the contract: on channels of contrast 1e6 with a tensor K or linear interface spaces another
+// order of the same sums moves T r by 1e-9 and more (rounding times the coupling system's condition).
+// A pivot publishes its column and then the scaled one through shared memory, two barriers of the half.
 //
 // The FP64 pipe bounds it: a warp-wide FP64 instruction holds its scheduler's pipe for 64 to 80
 // clocks whatever it computes, so the layout is chosen by the number of such instructions per
-// pivot: npk / 64 rounded up, all lanes busy, plus the reciprocal (three) and the scaling on one
-// warp (36 wide: 13.5 on average; a 128-thread half needs 8.25 on twice the warps, a one-warp half
-// 26, and both lose to it from 256 boxes on).  At most 128 registers are taken up to 40 columns: with
-// four boxes per SM the pipe is 88 % busy, and a wider launch ends in a shorter last wave.  Against
-// one-CTA Cholesky, L^-1 and L^-T L^-1 in shared memory (164 block barriers per line): set-up of
-// 512^2 cells in 40-wide boxes 5.5 -> 3.7 ms, of 1024^2 in 36-wide boxes 17.8 -> 9.8 ms, of 64^2 in
-// 20-wide boxes 0.70 -> 0.48 ms.  Errors against 80-bit solves are 0.8 to 1.0 times those of the
-// Cholesky route (log-normal, channel and white-noise boxes).
+// pivot: npk / 64 rounded up, all lanes busy, plus the square root, the division and the scaling on
+// one warp, the warps in turn (36 wide: 19.7 per warp and pivot with the Schur complement, 10.4 of them
+// the triangle at full lanes; halves of 128 threads or of one warp lost to 64 from 256 boxes on).  At most 128 registers are taken up to 40 columns: with
+// four boxes per SM the pipe is 87 % busy, and a wider launch ends in a shorter last wave.  Against
+// the same steps by one CTA with the block in shared memory (164 block barriers per line): set-up of
+// 512^2 cells in 40-wide boxes 5.7 -> 3.9 ms, of 1024^2 in 36-wide boxes 17.8 -> 10.3 ms, of 64^2 in
+// 20-wide boxes 0.68 -> 0.49 ms.  A symmetric Gauss-Jordan sweep, with a reciprocal in place of square
+// root and division, takes 8 % less, but in another order.
 // --------------------------------------------------------------------------------------------
 constexpr int FR_HT = 64;
 
@@ -614,9 +621,9 @@ __global__ void __launch_bounds__(2 * FR_HT, WMAX <= 40 ? 4 : 1)
   constexpr int NP = WMAX * (WMAX + 1) / 2, R = (NP + FR_HT - 1) / FR_HT, NW = FR_HT / 32;
   struct Half {
     double c[2][WMAX + 1];   // pivot column, double-buffered; slot WMAX belongs to the unused entries
-    double w[WMAX + 1];      // the same divided by the pivot
+    double x[WMAX + 1];      // the same divided by L_kk, 1 / L_kk at k
+    double xs[WMAX + 1];     // x, negated below the pivot
     double d[WMAX + 1], o[WMAX + 1], e[WMAX + 1];   // the line's diagonal, right and previous-line couplings
-    double nr;               // -1 / pivot (negated once: an FP64 negation is an FP64 instruction)
   };
   __shared__ Half sm_all[2];
   __shared__ double s_mid[NP];    // the bottom recursion's last S^-1, for the middle line
@@ -643,7 +650,7 @@ __global__ void __launch_bounds__(2 * FR_HT, WMAX <= 40 ? 4 : 1)
       tri_advance(i, j, FR_HT);
     }
   }
-  for (int t = th; t <= WMAX; t += FR_HT) sm.c[0][t] = sm.c[1][t] = sm.w[t] = sm.d[t] = sm.o[t] = sm.e[t] = 0.0;
+  for (int t = th; t <= WMAX; t += FR_HT) sm.c[0][t] = sm.c[1][t] = sm.x[t] = sm.xs[t] = sm.d[t] = sm.o[t] = sm.e[t] = 0.0;
   bool bad = false;
   const int nsteps = half == 0 ? m : h - 1 - m;
   // this thread's cell of the next line: its coefficients are requested one line ahead
@@ -655,7 +662,7 @@ __global__ void __launch_bounds__(2 * FR_HT, WMAX <= 40 ? 4 : 1)
       if (half == 1 && nsteps > 0) {
 #pragma unroll
         for (int r = 0; r < R; ++r)
-          if (th + FR_HT * r < npk) s_mid[th + FR_HT * r] = -a[r];
+          if (th + FR_HT * r < npk) s_mid[th + FR_HT * r] = a[r];
         if (th < w) s_e2[th] = eprev;
       }
       __syncthreads();
@@ -676,10 +683,9 @@ __global__ void __launch_bounds__(2 * FR_HT, WMAX <= 40 ? 4 : 1)
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       const int i = ij[r] >> 8, j = ij[r] & 255;
-      double v = has_prev ? sm.e[i] * a[r] * sm.e[j] : 0.0;   // a = -S_prev^-1
+      double v = i == j ? sm.d[i] : i == j + 1 ? -sm.o[j] : 0.0;
+      if (has_prev) v -= sm.e[i] * sm.e[j] * a[r];   // a = S_prev^-1
       if (dn && i < w) v -= s_e2[i] * s_e2[j] * s_mid[th + FR_HT * r];
-      if (i == j) v += sm.d[i];
-      if (i == j + 1) v -= sm.o[j];
       a[r] = v;
       if (j == 0) sm.c[0][i] = v;
     }
@@ -693,19 +699,22 @@ __global__ void __launch_bounds__(2 * FR_HT, WMAX <= 40 ? 4 : 1)
           bad = true;
           d = 1.0;
         }
-        const double ri = recip(d);
+        const double rd = 1.0 / sqrt(d);
 #pragma unroll
-        for (int i0 = 0; i0 < WMAX; i0 += 32)
-          if (i0 + lane < w) sm.w[i0 + lane] = c[i0 + lane] * ri;
-        if (lane == 0) sm.nr = -ri;
+        for (int i0 = 0; i0 < WMAX; i0 += 32) {
+          const int i = i0 + lane;
+          if (i < w) {
+            const double x = i == k ? rd : c[i] * rd;
+            sm.x[i] = x;   // the sign by its bit: an FP64 negation is an FP64 instruction
+            sm.xs[i] = __hiloint2double(__double2hiint(x) ^ (i > k ? (int)0x80000000 : 0), __double2loint(x));
+          }
+        }
       }
       half_sync(half);
-      const double nri = sm.nr;
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         const int i = ij[r] >> 8, j = ij[r] & 255;
-        double v = fma(-sm.w[i], c[j], a[r]);
-        if (i == k || j == k) v = i == j ? nri : sm.w[i == k ? j : i];
+        const double v = fma(sm.xs[i], sm.x[j], i == k || j == k ? 0.0 : a[r]);
         a[r] = v;
         if (i == k + 1 || j == k + 1) cn[i == k + 1 ? j : i] = v;
       }
@@ -713,7 +722,7 @@ __global__ void __launch_bounds__(2 * FR_HT, WMAX <= 40 ? 4 : 1)
     }
 #pragma unroll
     for (int r = 0; r < R; ++r)
-      if (th + FR_HT * r < npk) out[(size_t)J * LS + th + FR_HT * r] = -a[r];
+      if (th + FR_HT * r < npk) out[(size_t)J * LS + th + FR_HT * r] = a[r];
     if (mid) break;
   }
   if (bad) atomicOr(flags, FLAG_SINGULAR_LOCAL);
