@@ -77,18 +77,6 @@ __device__ __forceinline__ void grid_reduce(double (&v)[NV], double* partials, u
   if (threadIdx.x == 0) *counter = 0u;
 }
 
-// 1 / d from the hardware's reciprocal estimate (about 20 bits) by one cubic step,
-// r <- r + r (e + e^2) with e = 1 - d r: three dependent FMAs (within 2.3e-16 of 1 / d).  A result
-// outside the normal range takes the division.
-__device__ __forceinline__ double recip(double d) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
-  const double e = fma(-d, r, 1.0);
-  const double v = fma(r, fma(e, e, e), r);
-  const int ex = __double2hiint(v) & 0x7ff00000;   // integer tests: FP64 compares would take the FP64 pipe
-  return ex != 0 && ex != 0x7ff00000 ? v : 1.0 / d;
-}
-
 // Two-point-flux pieces (Sec. 3): half transmissibility tau = 2 K |f| / h_a.
 __device__ __forceinline__ double half_trans(double k, double area, double ha) { return 2.0 * k * area / ha; }
 

@@ -593,7 +593,8 @@ __global__ void __launch_bounds__(64) k_factor_sweep(Geo g, int kind, int LS, fl
 // clocks whatever it computes, so the layout is chosen by the number of such instructions per
 // pivot: npk / 64 rounded up, all lanes busy, plus the square root, the division and the scaling on
 // one warp, the warps in turn (36 wide: 19.7 per warp and pivot with the Schur complement, 10.4 of them
-// the triangle at full lanes; halves of 128 threads or of one warp lost to 64 from 256 boxes on).  At most 128 registers are taken up to 40 columns: with
+// the triangle at full lanes; halves of 128 threads or of one warp lost to 64 from 256 boxes on).  At most 128
+// registers are taken up to 40 columns: with
 // four boxes per SM the pipe is 87 % busy, and a wider launch ends in a shorter last wave.  Against
 // the same steps by one CTA with the block in shared memory (164 block barriers per line): set-up of
 // 512^2 cells in 40-wide boxes 5.7 -> 3.9 ms, of 1024^2 in 36-wide boxes 17.8 -> 10.3 ms, of 64^2 in

@@ -35,6 +35,10 @@ __device__ __forceinline__ bool nonzero_finite(double d) {
   const unsigned long long b = mag(d);
   return b != 0 && b != 0x7ff0000000000000ULL;
 }
+// -v by its sign bit
+__device__ __forceinline__ double flip_sign(double v) {
+  return __hiloint2double(__double2hiint(v) ^ (int)0x80000000, __double2loint(v));
+}
 // the largest magnitude across the CTA into a maximum in global memory
 __device__ __forceinline__ void cta_max_to(unsigned long long v, unsigned long long* dst) {
   for (int o = 16; o > 0; o >>= 1) {
@@ -46,8 +50,8 @@ __device__ __forceinline__ void cta_max_to(unsigned long long v, unsigned long l
 
 // One MF_TILE x MF_TILE tile of C (rows x cols of it) = (acc ? C : 0) + alpha A (rows x K) B (K x cols),
 // row-major operands with leading dimensions in global memory, one output per thread of the CTA; both
-// operands are staged in shared memory (sm: MF_TILE (2 K + 1) + K doubles).  Returns the magnitude of the
-// entry written.
+// operands are staged in shared memory (sm: MF_TILE (2 K + 1) + K doubles).  Each output is one sum in
+// increasing k.  Returns the magnitude of the entry written.
 __device__ unsigned long long cta_tile(int rows, int cols, int K, const double* A, int lda, const double* B, int ldb, double* C, int ldc,
                            double alpha, bool acc, double* sm) {
   double* As = sm;                            // [MF_TILE][K + 1]
@@ -63,14 +67,9 @@ __device__ unsigned long long cta_tile(int rows, int cols, int K, const double* 
   const bool on = r < rows && c < cols;
   const double old = on && acc ? C[(size_t)r * ldc + c] : 0.0;
   __syncthreads();
-  double s0 = 0.0, s1 = 0.0;
-  int k = 0;
-  for (; k + 1 < K; k += 2) {
-    s0 = fma(As[r * (K + 1) + k], Bs[k * MF_TILE + c], s0);
-    s1 = fma(As[r * (K + 1) + k + 1], Bs[(k + 1) * MF_TILE + c], s1);
-  }
-  if (k < K) s0 = fma(As[r * (K + 1) + k], Bs[k * MF_TILE + c], s0);
-  const double v = fma(alpha, s0 + s1, old);
+  double s = 0.0;
+  for (int k = 0; k < K; ++k) s = fma(As[r * (K + 1) + k], Bs[k * MF_TILE + c], s);
+  const double v = fma(alpha, s, old);
   if (on) C[(size_t)r * ldc + c] = v;
   return on ? mag(v) : 0ULL;
 }
@@ -80,12 +79,12 @@ __device__ __forceinline__ unsigned long long* mf_stats(const MfDev& m) {
 }
 
 // Gauss-Jordan inversion in registers of np rows by nc columns [c0, c0 + nc) of the pivot block (entry
-// t = thread + MF_THREADS r of the nc-wide rows; pivot k takes w_i = a_ik / a_kk and the row a_k., then a_ij -= w_i a_kj
-// off row and column k, row k = a_kj / a_kk, column k = -w_i, a_kk = 1 / a_kk).  The column is published by the
-// step before, over the whole block, the row by this CTA.  Bound by the FP64 pipe of its SM: an update is one FMA
-// per entry with every lane busy, the reciprocal and the scaled column cost a handful per warp, and the column is
-// kept negated because an FP64 negation per entry is an FP64 instruction too (with that and a division a pivot of
-// a 48-wide block took 2.0 us; now 1.6).
+// t = thread + MF_THREADS r of the nc-wide rows; pivot k takes the scaled row r_j = a_kj / a_kk and the column
+// c_i = a_ik, then a_ij -= c_i r_j off row and column k, row k = r_j, column k = -c_i / a_kk, a_kk = 1 / a_kk).  The
+// column is published by the step before, over the whole block, the row by this CTA.  Bound by the FP64 pipe of its
+// SM: an update is one FMA per entry with every lane busy, the division and the scaled row and column cost a handful
+// per warp, and the column is published with its sign flipped by an integer operation because an FP64 negation per
+// entry is an FP64 instruction too.
 template <int R>
 struct GjBlock {
   double a[R];
@@ -113,29 +112,29 @@ struct GjBlock {
     for (int r = 0; r < R; ++r)
       if ((ij[r] >> 8) < np) F[(size_t)(ij[r] >> 8) * f + (ij[r] & 255)] = a[r];
   }
-  // row and column k (own column kc, or none if outside) into the published arrays
+  // row and column k, this one negated (own column kc, or none if outside), into the published arrays
   __device__ __forceinline__ void publish(int k, int kc, double* row, double* col) const {
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       const int i = ij[r] >> 8, j = ij[r] & 255;
       if (i == k) row[j] = a[r];
-      if (j == kc) col[i] = a[r];
+      if (j == kc) col[i] = flip_sign(a[r]);
     }
   }
-  // pivot k with nw (the scaled column, negated), row k, row k times rp (1 / pivot); publishes row and column k + 1
-  __device__ __forceinline__ void pivot(int k, int kc, const double* nw, const double* row, const double* rowr, double rp,
+  // pivot k with nc (the column, negated), w (nc times rp), rowr (the row times rp) and rp (1 / pivot); publishes row
+  // and column k + 1
+  __device__ __forceinline__ void pivot(int k, int kc, const double* nc, const double* w, const double* rowr, double rp,
                                         double* next_row, double* next_col) {
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       if (r >= nr) break;
       const int i = ij[r] >> 8, j = ij[r] & 255;
-      const double ci = nw[i];
-      double v = fma(ci, row[j], a[r]);
+      double v = fma(nc[i], rowr[j], a[r]);
       if (i == k) v = j == kc ? rp : rowr[j];
-      else if (j == kc) v = ci;
+      else if (j == kc) v = w[i];
       a[r] = v;
       if (i == k + 1) next_row[j] = v;
-      if (j == kc + 1) next_col[i] = v;
+      if (j == kc + 1) next_col[i] = flip_sign(v);
     }
   }
 };
@@ -170,6 +169,12 @@ __global__ void __launch_bounds__(MF_THREADS) k_mf_gather(MfDev m, int first) {
   }
 }
 
+// The entry of a child's S that belongs to its message slots (row, column)
+__device__ __forceinline__ double schur_entry(const MfDev& m, const MfFront& ch, int row, int col) {
+  const int fc = ch.np + ch.nu;
+  return m.F[ch.fo + (size_t)(ch.np + row - ch.wo) * fc + ch.np + col - ch.wo];
+}
+
 // One CTA per front of a level: the original entries of the pivot rows and columns, and F11^-1 of the blocks that
 // one CTA inverts.
 template <int R>
@@ -180,30 +185,42 @@ __global__ void __launch_bounds__(MF_THREADS) k_mf_front(MfDev m, const double* 
   const MfFront fr = m.fr[fid];
   const int np = fr.np, nu = fr.nu, f = np + nu;
   double* __restrict__ F = m.F + fr.fo;
-  // the original entries on top of the children's (k_mf_gather), in batches of AB per thread, every load of a batch
-  // issued before its stores (the positions are distinct)
+  // the original entries with the children's (k_mf_gather), in batches of AB per thread, every load of a batch
+  // issued before its stores (the positions are distinct).  An entry is (original + first child) + second child:
+  // where both children have one, they are read again and added in that order.
   constexpr int AB = 8;
+  MfFront ch[2] = {};
+  for (int c = 0; c < 2; ++c)
+    if (fr.nch == 2) ch[c] = m.fr[fr.ch[c]];
   unsigned long long amax = 0;
   for (int t0 = threadIdx.x; t0 < fr.na; t0 += AB * MF_THREADS) {
     int dst[AB];
-    double v[AB], o[AB];
+    double v[AB], o[AB], o2[AB];
 #pragma unroll
     for (int e = 0; e < AB; ++e) {
       const int t = t0 + e * MF_THREADS;
       dst[e] = -1;
-      v[e] = 0.0;
+      v[e] = o[e] = o2[e] = 0.0;
       if (t < fr.na) {
         const int2 p = m.asmv[fr.ao + t];
         dst[e] = p.x;
         v[e] = ab[p.y];
+        bool both = false;
+        if (fr.nch == 2) {
+          const int2 si = m.inv[fr.io + p.x / f], sj = m.inv[fr.io + p.x % f];
+          both = si.x >= 0 && sj.x >= 0 && si.y >= 0 && sj.y >= 0;
+          if (both) {
+            o[e] = schur_entry(m, ch[0], si.x, sj.x);
+            o2[e] = schur_entry(m, ch[1], si.y, sj.y);
+          }
+        }
+        if (!both) o[e] = F[p.x];
       }
     }
 #pragma unroll
-    for (int e = 0; e < AB; ++e) o[e] = dst[e] >= 0 ? F[dst[e]] : 0.0;
-#pragma unroll
     for (int e = 0; e < AB; ++e)
       if (dst[e] >= 0) {
-        F[dst[e]] = o[e] + v[e];
+        F[dst[e]] = (v[e] + o[e]) + o2[e];
         const unsigned long long b = mag(v[e]);
         amax = b > amax ? b : amax;
       }
@@ -218,8 +235,8 @@ __global__ void __launch_bounds__(MF_THREADS) k_mf_front(MfDev m, const double* 
   // F11^-1 (at most R MF_THREADS entries: the launcher picks R by the level's largest block)
   const int tid = threadIdx.x;
   double* row = smd;                      // [2][np + 1] row k, double-buffered
-  double* col = row + 2 * (np + 1);       // [2][np + 1] column k
-  double* w = col + 2 * (np + 1);         // [np + 1] column k / pivot, negated
+  double* col = row + 2 * (np + 1);       // [2][np + 1] column k, negated
+  double* w = col + 2 * (np + 1);         // [np + 1] column k / pivot (both negated)
   double* rowr = w + np + 1;              // [np + 1] row k / pivot
   double* s_r = rowr + np + 1;            // 1 / pivot
   for (int t = tid; t < 6 * (np + 1); t += MF_THREADS) smd[t] = 0.0;
@@ -232,18 +249,18 @@ __global__ void __launch_bounds__(MF_THREADS) k_mf_front(MfDev m, const double* 
   for (int k = 0; k < np; ++k) {
     const int c = (k & 1) * (np + 1), n = np + 1 - c;
     if (tid < np) {
-      double d = col[c + k];
+      double d = flip_sign(col[c + k]);
       if (!nonzero_finite(d)) {
         bad = true;
         d = 1.0;
       }
-      const double r = recip(d);
-      w[tid] = col[c + tid] * -r;
+      const double r = 1.0 / d;
+      w[tid] = col[c + tid] * r;
       rowr[tid] = row[c + tid] * r;
       if (tid == 0) *s_r = r;
     }
     __syncthreads();
-    blk.pivot(k, k, w, row + c, rowr, *s_r, row + n, col + n);
+    blk.pivot(k, k, col + c, w, rowr, *s_r, row + n, col + n);
     __syncthreads();
   }
   blk.store(F, f, np);
@@ -267,13 +284,14 @@ __global__ void __launch_bounds__(MF_THREADS, 1) k_mf_gj_cluster(MfDev m, int fi
   const int cw = np / MF_GJ_CL, c0 = q * cw;
   double* F = m.F + fr.fo;
   constexpr int R = MF_MAX_NP * MF_MAX_NP / MF_GJ_CL / MF_THREADS;
-  double* pub = smd;                   // [2][np + 1] the pivot column, published by its owner
-  double* w = pub + 2 * (np + 1);      // [np + 1] the same divided by the pivot, negated
+  double* pub = smd;                   // [2][np + 1] the pivot column, negated, published by its owner
+  double* nc = pub + 2 * (np + 1);     // [np + 1] this CTA's copy of it
+  double* w = nc + np + 1;             // [np + 1] the same divided by the pivot
   double* row = w + np + 1;            // [2][cw + 1] this CTA's part of the pivot row
   double* rowr = row + 2 * (cw + 1);   // [cw + 1] the same divided by the pivot
   double* s_r = rowr + cw + 1;         // 1 / pivot
   const int tid = threadIdx.x;
-  for (int t = tid; t < 3 * (np + 1) + 3 * (cw + 1); t += MF_THREADS) smd[t] = 0.0;
+  for (int t = tid; t < 4 * (np + 1) + 3 * (cw + 1); t += MF_THREADS) smd[t] = 0.0;
   GjBlock<R> blk;
   blk.load(F + c0, f, np, cw);
   __syncthreads();
@@ -285,19 +303,20 @@ __global__ void __launch_bounds__(MF_THREADS, 1) k_mf_gj_cluster(MfDev m, int fi
     cl.sync();
     const double* rp = cl.map_shared_rank(pub + c * (np + 1), owner);
     if (tid < np) {   // np <= MF_MAX_NP < MF_THREADS
-      double d = rp[k];
+      double d = flip_sign(rp[k]);
       const double ci = rp[tid];
       if (!nonzero_finite(d)) {
         bad = true;
         d = 1.0;
       }
-      const double r = recip(d);
-      w[tid] = ci * -r;
+      const double r = 1.0 / d;
+      nc[tid] = ci;
+      w[tid] = ci * r;
       if (tid < cw) rowr[tid] = row[c * (cw + 1) + tid] * r;
       if (tid == 0) *s_r = r;
     }
     __syncthreads();
-    blk.pivot(k, kc, w, row + c * (cw + 1), rowr, *s_r, row + n * (cw + 1), pub + n * (np + 1));
+    blk.pivot(k, kc, nc, w, rowr, *s_r, row + n * (cw + 1), pub + n * (np + 1));
   }
   cl.sync();   // no CTA leaves while another may still read its published column
   blk.store(F + c0, f, np);
@@ -375,7 +394,7 @@ cudaError_t launch_mf_factor(const MfDev& m, const Plan& P, const double* ab, in
 #undef MRCM_MF_FRONT
       count_launch(1);
       if (big) {
-        const size_t sm_gj = 8 * (3 * (np_max + 1) + 3 * (np_max / MF_GJ_CL + 1) + 1);
+        const size_t sm_gj = 8 * (4 * (np_max + 1) + 3 * (np_max / MF_GJ_CL + 1) + 1);
         cudaError_t e2 = raise_smem_limit<k_mf_gj_cluster>();
         if (e2 != cudaSuccess) return e2;
         cudaLaunchConfig_t cfg = {};
@@ -411,32 +430,29 @@ cudaError_t launch_mf_factor(const MfDev& m, const Plan& P, const double* ab, in
   return cudaGetLastError();
 }
 
-// y_r = sum_k A[r][k] x[k] for r < rows (A row-major with leading dimension lda, in shared or global
-// memory): tpr threads per row (a power of two up to a warp, as many as the CTA has for the rows), each
-// with four partial sums over its columns k = q, q + tpr, ..., then the tpr sums in a fixed shuffle
-// order; emit(r, y) by the first thread of the row.  Deterministic.
+// y_r = sum_k A[r][k] x[k] for r < rows (A row-major with leading dimension lda, in shared or global memory), for
+// some rows of a front's block of `all` rows.  Every row is 4 d sums (d, a power of two up to 8, as many as the CTA
+// would have threads for all rows): chain (q, c) takes the columns q + (c + 4 i) d of the whole groups of four, and
+// (q, 0) the up to three left over; then c in pairs, then q in the order of a butterfly.  One chain per thread.  d
+// depends on the front alone, so a front cut into parts gives the bits of the whole one.  emit(r, y) by the first
+// thread of the row.
 template <class Emit>
-__device__ __forceinline__ void mf_rows(const double* A, int lda, int rows, int cols, const double* x, Emit emit) {
-  int tpr = 1;
-  while (tpr < 32 && tpr * 2 * rows <= MF_THREADS) tpr *= 2;
-  const int q = threadIdx.x % tpr, per = MF_THREADS / tpr;
+__device__ __forceinline__ void mf_rows(const double* A, int lda, int rows, int all, int cols, const double* x, Emit emit) {
+  int d = 1;
+  while (d < 8 && d * 2 * all <= MF_THREADS) d *= 2;
+  const int tpr = 4 * d, c = threadIdx.x & 3, q = (threadIdx.x >> 2) & (d - 1), per = MF_THREADS / tpr;
   for (int r0 = 0; r0 < rows; r0 += per) {
     const int r = r0 + threadIdx.x / tpr;
-    double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+    double s = 0.0;
     if (r < rows) {
       const double* a = A + (size_t)r * lda;
       int k = q;
-      for (; k + 3 * tpr < cols; k += 4 * tpr) {
-        s0 = fma(a[k], x[k], s0);
-        s1 = fma(a[k + tpr], x[k + tpr], s1);
-        s2 = fma(a[k + 2 * tpr], x[k + 2 * tpr], s2);
-        s3 = fma(a[k + 3 * tpr], x[k + 3 * tpr], s3);
-      }
-      for (; k < cols; k += tpr) s0 = fma(a[k], x[k], s0);
+      for (; k + 3 * d < cols; k += 4 * d) s = fma(a[k + c * d], x[k + c * d], s);
+      if (c == 0)
+        for (; k < cols; k += d) s = fma(a[k], x[k], s);
     }
-    double t = (s0 + s1) + (s2 + s3);
-    for (int o = 1; o < tpr; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    if (r < rows && q == 0) emit(r, t);
+    for (int o = 1; o < tpr; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (r < rows && c == 0 && q == 0) emit(r, s);
   }
 }
 
@@ -481,13 +497,13 @@ __device__ __forceinline__ double msg_get(const uint4* slot, unsigned E, int* fl
 // entry for a current one.  All CTAs are resident, and each takes its parts in increasing level
 // (decreasing, backward), so every wait ends; the waits are bounded all the same.  What a part reads
 // besides (its rows of B or [F11^-1 D], copied into shared memory, its slots) is requested before it
-// waits.  Rows are dotted by up to a warp each, in a fixed order, so the result is deterministic.
+// waits.  Rows are dotted by up to a warp each, in an order that does not depend on the parts.
 //
 // The dependence chain bounds it: 2 x levels hand-overs, each a write, a poll and a short product.  With
 // the whole front on one CTA the upper levels' products alone took 2.4 to 4.7 us there (128 x 128 FMA at
 // 1.6 a clock), and a completion flag per front cost a fence, a poll by one thread and a second read:
-// 131 us on 64 x 64 subdomains (9 levels), 80 us on 32 x 32, 56 us on 16 x 16, with the right-hand side
-// formed by a launch of its own; now 60, 39 and 25 us.
+// 134 us on 64 x 64 subdomains (9 levels), 76 us on 32 x 32, 49 us on 16 x 16, with the right-hand side
+// formed by a launch of its own; now 60, 34 and 23 us.
 __global__ void __launch_bounds__(MF_THREADS, 2) k_mf_solve(MfDev m, const double* __restrict__ mom0,
                                                          double* __restrict__ g, int* flags, int mcap) {
   extern __shared__ __align__(16) double smd[];
@@ -524,7 +540,7 @@ __global__ void __launch_bounds__(MF_THREADS, 2) k_mf_solve(MfDev m, const doubl
     }
     cp_async_wait_all();
     __syncthreads();
-    mf_rows(staged ? M : Bx, staged ? np + 1 : np, rows, np, v,
+    mf_rows(staged ? M : Bx, staged ? np + 1 : np, rows, fr.nu, np, v,
             [&](int r, double t) { msg_put(m.W + fr.wo + w.u0 + r, v[np + r] - t, E); });
     __syncthreads();
   }
@@ -538,7 +554,7 @@ __global__ void __launch_bounds__(MF_THREADS, 2) k_mf_solve(MfDev m, const doubl
       v[t] = t < np ? m.V[w.vo + t] : -msg_get(m.X + m.idx[fr.io + t], E, flags);
     cp_async_wait_all();
     __syncthreads();
-    mf_rows(staged ? M : F, staged ? f + 1 : f, rows, f, v, [&](int r, double t) {
+    mf_rows(staged ? M : F, staged ? f + 1 : f, rows, np, f, v, [&](int r, double t) {
       const int u = m.idx[fr.io + w.p0 + r];
       msg_put(m.X + u, t, E);
       g[u] = t;

@@ -89,3 +89,14 @@ def test_local_factors(case):
     """Side moments of the basis functions: boundary problems on both kinds of boxes."""
     from paper_2606_08883_gb300 import mrcm
     check(case, "moments", solver(case).debug(mrcm.MRCM_DBG_MOMENTS))
+
+
+@pytest.mark.parametrize("case", list(CASES))
+def test_coupling_system(case):
+    """Interface coefficients and T r: assembly, elimination and products of the fronts, their solves."""
+    import torch
+    from paper_2606_08883_gb300 import mrcm
+    s = solver(case)
+    z = s.apply_precond(torch.as_tensor((integers(s.n, 3) - (1 << 19)) / float(1 << 19), device="cuda"))
+    check(case, "coupling", s.debug(mrcm.MRCM_DBG_COARSE))
+    check(case, "precond", z.cpu().numpy())
