@@ -378,8 +378,8 @@ NCU_TRAFFIC = {
 # The Arnoldi step's traffic grows with the inner step j: (bytes, j) of the captured launch, scaled
 # to the solve's average launch by the model's algorithmic bytes (krylov_model), in which the basis
 # sweeps that make the traffic grow in proportion.
-NCU_TRAFFIC_KRYLOV = (576.339968e6 + 62.4448e6, 5, "paper_2606_08883_gb300/csrc/k_krylov.cu",
-                      "3621efcce9df04e1d32efe245a1936f6023331f078e795b1fc83a4f8182da5be")
+NCU_TRAFFIC_KRYLOV = (576.625664e6 + 62.182912e6, 5, "paper_2606_08883_gb300/csrc/k_krylov.cu",
+                      "158ea8b9bb392cc3614d463ccfbdca86f9b5347239b3d3fc589a15a482b634f3")
 
 
 def krylov_traffic(n, iterations, restart):

@@ -147,8 +147,8 @@ __global__ void __launch_bounds__(RED_THREADS) k_residual_norm(Geo g, const doub
 
 // ============================================================================================
 // Cooperative Arnoldi step.  All blocks are co-resident (cooperative launch); grid barriers are
-// an arrival counter plus a generation word, polled with a bounded spin that sets FLAG_TIMEOUT and
-// returns instead of waiting forever.
+// a counter that only grows, polled with a bounded spin that sets FLAG_TIMEOUT and returns instead of
+// waiting forever.
 // ============================================================================================
 // One Arnoldi step (inner step j) in a single cooperative launch, with the modified
 // Gram-Schmidt coefficients obtained from one global reduction.  MGS computes
@@ -158,13 +158,17 @@ __global__ void __launch_bounds__(RED_THREADS) k_residual_norm(Geo g, const doub
 // h_i = (T a)_i for i < j is a product instead of a sequential solve, and the last coefficient is
 // the MGS recurrence itself, h_j = a_j - sum_k r_k h_k.
 //
+// A dot product's order is part of the contract: slices of arn_grid, each summed over its warps' parts in
+// part order, then the slices.  On channels of contrast 1e6 another cut of the same vectors moves a converged
+// p by up to 3e-8 (one solve in 200 by more than 1e-9).
+//
 // Barriers: arrivals add to a counter that only grows (a multiple of the grid's CTAs between launches;
 // zeroed with the flags at each set-up), so a barrier is one release and one acquire poll, and work that
 // only the last block needs (the rotations) runs between its arrival and its wait.  Vectors of up to
 // ARN_CLUSTER_N elements take one cluster of up to eight CTAs and the cluster's hardware barrier instead;
-// with few CTAs every one forms all totals itself and the second barrier goes.  With the finer cut of
-// arn_grid a step takes 34.8 -> 25.4 us at 64^2, 37.7 -> 27.7 at 128^2, 47.4 -> 43.0 at 512^2, 87.3 -> 83.3 at
-// 1024^2 (the FP64 pipe's share of it 1, 2, 18 and 72 us).
+// with few CTAs every one forms all totals itself and the second barrier goes.  Against three barriers with
+// a generation word each a step takes 36.4 -> 29.6 us at 64^2, 37.0 -> 33.3 at 128^2, 38.7 -> 35.1 at 256^2,
+// 46.5 -> 43.0 at 512^2, 87.2 -> 84.1 at 1024^2 (the FP64 pipe's share of the last two 18 and 72 us).
 //
 // Per step: one sweep over the basis that forms a_k and r_k together for every k < j (one read of
 // v_k), plus (w, v_j) and ||A z_j||^2; one sweep for w -= V h and ||w||^2; three grid barriers.
@@ -180,7 +184,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_residual_norm(Geo g, const doub
 //    coefficients h come from on-chip data;
 //  * the previous rotations of the Hessenberg column are a first-order linear recurrence
 //    (y_{i+1} = -s_i y_i + c_i h_{i+1}) and are applied by a warp-wide scan in the last block,
-//    overlapped with its share of the update sweep.
+//    between its last arrival and its wait.
 // Cross-block sums are taken in block order (deterministic).
 struct LsArgs {
   const double* z;      // z_j
@@ -207,9 +211,9 @@ constexpr int DOT_UNROLL = 4;   // elements of the swept basis vector in flight 
 constexpr int UPD_EL = 2;       // vector elements per thread in the update sweep
 constexpr int UPD_UU = 2;       // basis vectors per ring stage
 constexpr int UPD_DS = 3;       // ring stages
-constexpr int ARN_CHUNK = 256;        // fewest elements per CTA
+constexpr int ARN_CHUNK = ARN_THREADS;   // fewest elements per CTA
 constexpr int ARN_CLUSTER = 8;        // most CTAs of the one-cluster form
-constexpr int ARN_CLUSTER_N = ARN_CLUSTER * 512;   // elements up to which it is taken
+constexpr int ARN_CLUSTER_N = ARN_CLUSTER * ARN_CHUNK;   // elements up to which it is taken
 constexpr int ARN_DIRECT = 32;        // CTAs up to which every CTA forms all totals
 constexpr int ROW_TPR = 4;      // threads per row of T in the coefficient product
 constexpr int ARN_SMALL = 5 * 264;                               // a | r | h | cs | sn (doubles)
@@ -472,18 +476,13 @@ __global__ void __launch_bounds__(ARN_THREADS, 1) k_arnoldi_ls(Geo g, LsArgs a) 
       if (lane == 16) s_dot[2 * warp + 1] = v;
     }
     __syncthreads();
-    // the parts' sums, a warp per sum where there are many parts, else a thread
-    for (int x = wpt > 6 ? warp : tid; x < 2 * nr; x += wpt > 6 ? nw : nt) {
-      const int uu = x >> 1, which = x & 1;
+    if (tid < 2 * nr) {   // the parts' sums, in part order
+      const int uu = tid >> 1, which = tid & 1;
       const int t = j - (u0 + uu);
       double acc = 0.0;
-      if (wpt > 6) {
-        acc = warp_sum(lane < wpt ? s_dot[2 * (uu * wpt + lane) + which] : 0.0);
-      } else {
-        for (int q = 0; q < wpt; ++q) acc += s_dot[2 * (uu * wpt + q) + which];
-      }
+      for (int q = 0; q < wpt; ++q) acc += s_dot[2 * (uu * wpt + q) + which];
       const int slot = which == 0 ? t : (t < j ? j + 1 + t : 2 * j + 1);
-      if (wpt <= 6 || lane == 0) a.part[(size_t)slot * G + b] = acc;
+      a.part[(size_t)slot * G + b] = acc;
     }
     __syncthreads();
   }
@@ -641,9 +640,10 @@ __global__ void __launch_bounds__(ARN_THREADS, 1) k_arnoldi_ls(Geo g, LsArgs a) 
   }
 }
 
-// CTAs for a vector of n elements: the FP64 pipe takes (3 j + 13) n operations per step, so vectors that
-// would leave SMs idle are cut finer than a thread per element (256^2 on 64 CTAs of 1,024 elements: 38.6 us
-// a step, on every SM: 29.4)
+// CTAs for a vector of n elements: one per SM, at least a thread's element each.  Slices of 256 elements take a
+// step alone from 29.6 to 25.5 us at 64^2 and from 35.1 to 29.5 at 256^2, but in another order of the sums, and a
+// burst of nine requests on eight streams from 13.3 to 15.0 ms: a small request's cooperative launch then waits
+// until every SM is free.
 static int arn_grid(int sms, size_t n) {
   return (int)std::max<size_t>(1, std::min<size_t>((size_t)sms, (n + ARN_CHUNK - 1) / ARN_CHUNK));
 }
@@ -681,12 +681,6 @@ cudaError_t launch_arnoldi(const Geo& g, const double* z, double* V, int j, size
   const int sms = occ.sms, per_sm = occ.per_sm;
   int grid = arn_grid(sms, n);
   const bool cluster = n <= (size_t)ARN_CLUSTER_N && occ.clusters > 0;
-  if (cluster)
-    for (int p = ARN_CLUSTER; p > 0; p >>= 1)   // the largest power of two up to the CTAs that have elements
-      if (grid >= p) {
-        grid = p;
-        break;
-      }
   if (grid > ARNOLDI_MAX_BLOCKS || per_sm < 1 || ldh > 257) return cudaErrorNotSupported;
   const size_t tri = (size_t)j * (j > 0 ? j - 1 : 0) / 2;
   const int stage_T = 8 * (ARN_SMALL + std::max<size_t>(ARN_RING, tri)) <= (size_t)ARN_SMEM_MAX ? 1 : 0;

@@ -100,3 +100,10 @@ def test_coupling_system(case):
     z = s.apply_precond(torch.as_tensor((integers(s.n, 3) - (1 << 19)) / float(1 << 19), device="cuda"))
     check(case, "coupling", s.debug(mrcm.MRCM_DBG_COARSE))
     check(case, "precond", z.cpu().numpy())
+
+
+@pytest.mark.parametrize("case", list(CASES))
+def test_solution(case):
+    """p of a whole solve, which the inner products of the Krylov basis enter too."""
+    p, info = solver(case).solve()
+    check(case, "solve", p.cpu().numpy())
