@@ -182,7 +182,7 @@ MfDev mfdev(mrcm_handle h) {
   m.item = at<MfItem>(h, L.mf_item);
   m.inv = at<int2>(h, L.mf_inv);
   m.rhs = at<int2>(h, L.mf_rhs);
-  m.W = at<uint4>(h, L.mf_msg);
+  m.W = at<ulonglong2>(h, L.mf_msg);
   m.X = m.W + P.mf_wslots;
   m.nitem = (int)P.mf_item.size();
   m.max_f = P.mf_max_f;

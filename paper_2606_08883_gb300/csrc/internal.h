@@ -336,8 +336,8 @@ struct MfDev {
   const int2* rhs;      // side moments of each unknown's right-hand side
   double* F;
   double* V;            // the parts' v_P
-  uint4* W;             // upward messages (w_U of every front)
-  uint4* X;             // solution entries as messages [2E nq]
+  ulonglong2* W;        // upward messages (w_U of every front)
+  ulonglong2* X;        // solution entries as messages [2E nq]
   unsigned* scr;        // [2, 6) two 8-byte maxima (|G| entries, |S| entries); [8] solve epoch,
                         // [9] CTAs finished in the current solve
   int nitem;

@@ -465,24 +465,24 @@ __device__ __forceinline__ void cp_async_wait_all() {
   asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
 }
 
-// Messages: a double in a 16-byte slot as two (half, epoch) pairs.  Each 8-byte pair is written and
-// read at once, so a slot whose two epochs are the solve's holds the solve's value, and no fence or
-// separate flag is needed.
-__device__ __forceinline__ void msg_put(uint4* slot, double v, unsigned E) {
-  asm volatile("st.volatile.global.v4.u32 [%0], {%1, %2, %3, %4};\n" ::"l"(slot), "r"((unsigned)__double2loint(v)), "r"(E),
-               "r"((unsigned)__double2hiint(v)), "r"(E)
+// Messages: a double in a 16-byte slot as two 64-bit words, each a half of it below the solve's epoch (the slots of
+// NCCL's LL protocol).  Each word is one access of the memory model, also in a vector of two (of four 32-bit
+// elements, as the slots were written before, every one is an access of its own, and a reader could take a new epoch
+// beside an old half).  So two words with the solve's epoch hold the solve's value whatever order they arrive in,
+// and no fence or separate flag is needed.
+__device__ __forceinline__ void msg_put(ulonglong2* slot, double v, unsigned E) {
+  const unsigned long long e = (unsigned long long)E << 32;
+  asm volatile("st.volatile.global.v2.u64 [%0], {%1, %2};\n" ::"l"(slot), "l"(e | (unsigned)__double2loint(v)),
+               "l"(e | (unsigned)__double2hiint(v))
                : "memory");
 }
 // Polls a slot.  The wait is bounded: when it gives up, here or in any other CTA (FLAG_TIMEOUT is set),
 // it returns 0 and the later waits of the launch give up after a few polls.
-__device__ __forceinline__ double msg_get(const uint4* slot, unsigned E, int* flags) {
+__device__ __forceinline__ double msg_get(const ulonglong2* slot, unsigned E, int* flags) {
   for (long long spins = 0; spins < BARRIER_SPIN_LIMIT; ++spins) {
-    unsigned lo, e0, hi, e1;
-    asm volatile("ld.volatile.global.v4.u32 {%0, %1, %2, %3}, [%4];\n"
-                 : "=r"(lo), "=r"(e0), "=r"(hi), "=r"(e1)
-                 : "l"(slot)
-                 : "memory");
-    if (e0 == E && e1 == E) return __hiloint2double((int)hi, (int)lo);
+    unsigned long long lo, hi;
+    asm volatile("ld.volatile.global.v2.u64 {%0, %1}, [%2];\n" : "=l"(lo), "=l"(hi) : "l"(slot) : "memory");
+    if ((unsigned)(lo >> 32) == E && (unsigned)(hi >> 32) == E) return __hiloint2double((int)hi, (int)lo);
     if ((spins & 1023) == 1023 && (*(volatile int*)flags & FLAG_TIMEOUT)) return 0.0;
   }
   atomicOr(flags, FLAG_TIMEOUT);
