@@ -378,8 +378,8 @@ NCU_TRAFFIC = {
 # The Arnoldi step's traffic grows with the inner step j: (bytes, j) of the captured launch, scaled
 # to the solve's average launch by the model's algorithmic bytes (krylov_model), in which the basis
 # sweeps that make the traffic grow in proportion.
-NCU_TRAFFIC_KRYLOV = (576.625664e6 + 62.182912e6, 5, "paper_2606_08883_gb300/csrc/k_krylov.cu",
-                      "158ea8b9bb392cc3614d463ccfbdca86f9b5347239b3d3fc589a15a482b634f3")
+NCU_TRAFFIC_KRYLOV = (576.487936e6 + 62.679296e6, 5, "paper_2606_08883_gb300/csrc/k_krylov.cu",
+                      "e099eb7516a47ab82e145cb0b416229ac51b754d7435b4700501d691d76d788f")
 
 
 def krylov_traffic(n, iterations, restart):

@@ -236,6 +236,9 @@ enum { MRCM_DBG_TRANS = 0, MRCM_DBG_PHI = 1, MRCM_DBG_PSI = 2, MRCM_DBG_MOMENTS 
        MRCM_DBG_COARSE = 5, MRCM_DBG_ZMRCM = 6 };
 mrcm_status mrcm_debug_get(mrcm_handle h, int32_t what, double* host_out, size_t cap, size_t* len,
                            void* stream);
+/* How often the coupling solve and the Arnoldi step of this handle poll before a wait gives up
+ * (0: the default, seconds of polling).  A small number makes their waits run out, to test what follows. */
+mrcm_status mrcm_debug_wait_limit(mrcm_handle h, int64_t polls);
 
 /* Per-phase device time.  While enabled, the library records a pair of CUDA events on the caller's
  * stream around every kernel group of a phase (events are created on the first use and reused).

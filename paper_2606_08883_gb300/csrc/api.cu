@@ -167,6 +167,8 @@ CoarseDev coarse(mrcm_handle h) {
   return c;
 }
 
+long long wait_polls(mrcm_handle h) { return h->wait_polls > 0 ? h->wait_polls : BARRIER_SPIN_LIMIT; }
+
 MfDev mfdev(mrcm_handle h) {
   MfDev m;
   const Layout& L = h->lay;
@@ -187,6 +189,7 @@ MfDev mfdev(mrcm_handle h) {
   m.nitem = (int)P.mf_item.size();
   m.max_f = P.mf_max_f;
   m.mcap = P.mf_mcap;
+  m.polls = wait_polls(h);
   return m;
 }
 
@@ -735,7 +738,7 @@ mrcm_status mrcm_gmres_solve(mrcm_handle h, const double* b, double* p, double* 
           cudaError_t ea = cudaErrorNotSupported;
           if (fused)
             ea = launch_arnoldi(g, zj, V, j, n, H, ldh, cs, sn, gv, slot, w, at<double>(h, L.apart),
-                                at<double>(h, L.atot), at<double>(h, L.aT), flags, st);
+                                at<double>(h, L.atot), at<double>(h, L.aT), flags, wait_polls(h), st);
           if (ea == cudaErrorNotSupported) {
             fused = false;
             (void)cudaGetLastError();
@@ -766,7 +769,7 @@ mrcm_status mrcm_gmres_solve(mrcm_handle h, const double* b, double* p, double* 
         ++it;
         if (slot->flags == STEP_PENDING || (slot->flags & FLAG_TIMEOUT)) {
           cudaStreamSynchronize(st);   // the step in flight writes the other slot
-          return fail(h, MRCM_ERR_TIMEOUT, "a bounded device wait gave up (Arnoldi grid barrier or local-solve line copy)");
+          return fail(h, MRCM_ERR_TIMEOUT, "a bounded device wait gave up (Arnoldi grid barrier, coupling solve or local-solve line copy)");
         }
         if (h->cancel && *h->cancel) {
           cudaStreamSynchronize(st);
@@ -906,6 +909,12 @@ mrcm_status mrcm_profile_read(mrcm_handle h, double* ms, int64_t* launches, int3
       h->ph_ms[i] = 0.0;
       h->ph_launch[i] = 0;
     }
+  return MRCM_OK;
+}
+
+mrcm_status mrcm_debug_wait_limit(mrcm_handle h, int64_t polls) {
+  if (!h || polls < 0) return fail(h, MRCM_ERR_INVALID_ARG, "null handle or a negative number of polls");
+  h->wait_polls = polls;
   return MRCM_OK;
 }
 

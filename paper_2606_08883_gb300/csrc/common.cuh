@@ -177,7 +177,6 @@ __device__ __forceinline__ int stencil_col0() { return (blockIdx.x * 4 + (thread
 // Grid-wide barrier for cooperative launches (every block co-resident).  bar[0] counts arrivals
 // (zero between barriers), bar[1] is the generation.  A block that polls more than
 // BARRIER_SPIN_LIMIT times sets FLAG_TIMEOUT in *flags and returns false instead of waiting on.
-constexpr long long BARRIER_SPIN_LIMIT = 1LL << 24;   // ~1-2 s of polling, then give up
 
 // Returns false if the wait gave up (the flag is set; the caller returns).
 __device__ __forceinline__ bool grid_barrier(unsigned* bar, int* flags) {

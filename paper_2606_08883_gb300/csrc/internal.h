@@ -188,6 +188,8 @@ struct StepReport {
 };
 constexpr int STEP_PENDING = -1;
 
+constexpr long long BARRIER_SPIN_LIMIT = 1LL << 24;   // polls of a device wait (seconds), then it gives up
+
 }  // namespace mrcm
 
 // The handle.
@@ -212,6 +214,7 @@ struct mrcm_ctx {
   int coarse_n;       // 2E
   std::vector<int> tab_host;  // plan tables uploaded to the device
   bool keep_z0 = false;       // keep the last multiscale solution for debug reads
+  long long wait_polls = 0;   // polls of the coupling solve's and the Arnoldi step's waits (0: the default)
   const volatile int* cancel = nullptr;  // set by the request server; checked once per GMRES step
   // phase profiler
   bool prof = false;
@@ -343,6 +346,7 @@ struct MfDev {
   int nitem;
   int max_f;            // largest front (np + nu)
   int mcap;             // doubles of front rows the solve stages in shared memory
+  long long polls;      // polls before a wait of the solve gives up
 };
 // Set-up: fronts level by level (assembly from the band copy of G and F11^-1, then the D and B
 // tiles, then the Schur-complement tiles) and a final growth check that sets FLAG_NOPIV_REJECTED
@@ -354,7 +358,7 @@ cudaError_t launch_mf_factor(const MfDev& m, const Plan& P, const double* ab, in
 cudaError_t launch_mf_solve(const MfDev& m, const double* mom0, double* g, int* flags, cudaStream_t st);
 cudaError_t launch_arnoldi(const Geo& g, const double* z, double* V, int j, size_t n, double* H, int ldh, double* cs,
                            double* sn, double* gv, StepReport* report, double* wbuf, double* part, double* tot, double* Tm,
-                           int* flags, cudaStream_t st);
+                           int* flags, long long polls, cudaStream_t st);
 
 // Krylov helpers (k_krylov.cu)
 cudaError_t launch_norm2(const double* x, size_t n, double* partials, unsigned* counter, double* out,

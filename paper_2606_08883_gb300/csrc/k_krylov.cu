@@ -163,7 +163,8 @@ __global__ void __launch_bounds__(RED_THREADS) k_residual_norm(Geo g, const doub
 // p by up to 3e-8 (one solve in 200 by more than 1e-9).
 //
 // Barriers: arrivals add to a counter that only grows (a multiple of the grid's CTAs between launches;
-// zeroed with the flags at each set-up), so a barrier is one release and one acquire poll, and work that
+// zeroed with the flags at each set-up; a launch that gave up leaves it between two multiples, and its status
+// in the flags, with which every later step fails until that set-up), so a barrier is one release and one acquire poll, and work that
 // only the last block needs (the rotations) runs between its arrival and its wait.  Vectors of up to
 // ARN_CLUSTER_N elements take one cluster of up to eight CTAs and the cluster's hardware barrier instead;
 // with few CTAs every one forms all totals itself and the second barrier goes.  Against three barriers with
@@ -203,6 +204,7 @@ struct LsArgs {
   double* Tm;           // (I + R)^-1, row-major lower, leading dimension ldh
   unsigned long long* bar;
   int* flags;
+  long long polls;      // polls before a barrier gives up
   int stage_T;          // 1: rows of T staged in shared memory (fits), 0: read from global
 };
 
@@ -338,6 +340,7 @@ template <bool CL>
 struct ArnBarrier {
   unsigned long long* count;
   int* flags;
+  long long polls;
   unsigned long long target = 0;   // thread 0: the count that completes the current barrier
   // thread 0, before its first arrival: fewer than gridDim.x arrivals of the launch can be in the count
   __device__ __forceinline__ void init() {
@@ -365,13 +368,14 @@ struct ArnBarrier {
     __shared__ int s_ok;
     if (threadIdx.x == 0) {
       s_ok = 0;
-      for (long long spins = 0; spins < BARRIER_SPIN_LIMIT; ++spins) {
+      for (long long spins = 0; spins < polls; ++spins) {
         unsigned long long c;
         asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(c) : "l"(count) : "memory");
         if (c >= target) {
           s_ok = 1;
           break;
         }
+        if ((spins & 1023) == 1023 && (*(volatile int*)flags & FLAG_TIMEOUT)) break;   // another wait gave up
       }
       if (!s_ok) atomicOr(flags, FLAG_TIMEOUT);
     }
@@ -394,7 +398,7 @@ __global__ void __launch_bounds__(ARN_THREADS, 1) k_arnoldi_ls(Geo g, LsArgs a) 
   const size_t lo = (size_t)b * chunk < n ? (size_t)b * chunk : n;
   const size_t hi = lo + chunk < n ? lo + chunk : n;
   double* w = a.wbuf;
-  ArnBarrier<CL> bar{a.bar, a.flags};
+  ArnBarrier<CL> bar{a.bar, a.flags, a.polls};
   bar.init();
   const double* vj = a.V + (size_t)j * n;
   double* ring = sh + ARN_SMALL;
@@ -651,7 +655,7 @@ static int arn_grid(int sms, size_t n) {
 // Returns cudaErrorNotSupported when one co-resident wave cannot cover the grid.
 cudaError_t launch_arnoldi(const Geo& g, const double* z, double* V, int j, size_t n, double* H, int ldh, double* cs,
                            double* sn, double* gv, StepReport* report, double* wbuf, double* part, double* tot, double* Tm,
-                           int* flags, cudaStream_t st) {
+                           int* flags, long long polls, cudaStream_t st) {
   struct Occ {
     int sms = 0, per_sm = 0, clusters = 0;
   };
@@ -687,7 +691,7 @@ cudaError_t launch_arnoldi(const Geo& g, const double* z, double* V, int j, size
   const size_t smem = 8 * (ARN_SMALL + (stage_T ? std::max<size_t>(ARN_RING, tri) : (size_t)ARN_RING));
   // the barrier's arrivals share the flag block, which each set-up zeroes (words 32, 33)
   LsArgs a{z, V, j, n, H, ldh, cs, sn, gv, report, wbuf, part, tot, Tm,
-           reinterpret_cast<unsigned long long*>(flags + 32), flags, stage_T};
+           reinterpret_cast<unsigned long long*>(flags + 32), flags, polls, stage_T};
   cudaError_t e;
   if (cluster) {
     cudaLaunchConfig_t cfg = {};

@@ -477,9 +477,10 @@ __device__ __forceinline__ void msg_put(ulonglong2* slot, double v, unsigned E) 
                : "memory");
 }
 // Polls a slot.  The wait is bounded: when it gives up, here or in any other CTA (FLAG_TIMEOUT is set),
-// it returns 0 and the later waits of the launch give up after a few polls.
-__device__ __forceinline__ double msg_get(const ulonglong2* slot, unsigned E, int* flags) {
-  for (long long spins = 0; spins < BARRIER_SPIN_LIMIT; ++spins) {
+// it returns 0, and the other waits of the launch give up at their 1,024th poll.  The CTA goes on with what it has
+// (every front's messages are written, with the current epoch), and the status word tells the host.
+__device__ __forceinline__ double msg_get(const ulonglong2* slot, unsigned E, int* flags, long long polls) {
+  for (long long spins = 0; spins < polls; ++spins) {
     unsigned long long lo, hi;
     asm volatile("ld.volatile.global.v2.u64 {%0, %1}, [%2];\n" : "=l"(lo), "=l"(hi) : "l"(slot) : "memory");
     if ((unsigned)(lo >> 32) == E && (unsigned)(hi >> 32) == E) return __hiloint2double((int)hi, (int)lo);
@@ -533,8 +534,8 @@ __global__ void __launch_bounds__(MF_THREADS, 2) k_mf_solve(MfDev m, const doubl
         const int2 o = m.rhs[m.idx[pos]];
         val = o.y >= 0 ? -(mom0[o.x] + mom0[o.y]) : -(mom0[o.x] - mom0[~o.y]);
       }
-      if (slot.x >= 0) val += msg_get(m.W + slot.x, E, flags);
-      if (slot.y >= 0) val += msg_get(m.W + slot.y, E, flags);
+      if (slot.x >= 0) val += msg_get(m.W + slot.x, E, flags, m.polls);
+      if (slot.y >= 0) val += msg_get(m.W + slot.y, E, flags, m.polls);
       v[t] = val;
       if (t < np) m.V[w.vo + t] = val;
     }
@@ -551,7 +552,7 @@ __global__ void __launch_bounds__(MF_THREADS, 2) k_mf_solve(MfDev m, const doubl
     const double* F = m.F + fr.fo + (size_t)w.p0 * f;
     const bool staged = stage(F, rows, f);
     for (int t = tid; t < f; t += MF_THREADS)
-      v[t] = t < np ? m.V[w.vo + t] : -msg_get(m.X + m.idx[fr.io + t], E, flags);
+      v[t] = t < np ? m.V[w.vo + t] : -msg_get(m.X + m.idx[fr.io + t], E, flags, m.polls);
     cp_async_wait_all();
     __syncthreads();
     mf_rows(staged ? M : F, staged ? f + 1 : f, rows, np, f, v, [&](int r, double t) {

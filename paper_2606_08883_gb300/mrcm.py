@@ -69,6 +69,7 @@ _SIGS = {
     "mrcm_plan_export": ([_P, _Q, C.POINTER(C.c_int32), C.c_size_t, C.POINTER(C.c_size_t)], C.c_int),
     "mrcm_plan_mf_export": ([_P, _Q, C.POINTER(C.c_int32), C.c_size_t, C.POINTER(C.c_size_t)], C.c_int),
     "mrcm_debug_get": ([_H, C.c_int32, C.c_void_p, C.c_size_t, C.POINTER(C.c_size_t), C.c_void_p], C.c_int),
+    "mrcm_debug_wait_limit": ([_H, C.c_int64], C.c_int),
     "mrcm_profile_enable": ([_H, C.c_int32], C.c_int),
     "mrcm_profile_select": ([_H, C.c_uint32, C.c_int32], C.c_int),
     "mrcm_profile_read": ([_H, C.POINTER(C.c_double), C.POINTER(C.c_int64), C.c_int32, C.c_int32, C.c_void_p], C.c_int),
