@@ -574,12 +574,10 @@ __global__ void __launch_bounds__(MF_THREADS, 2) k_mf_solve(MfDev m, const doubl
 }
 
 cudaError_t launch_mf_solve(const MfDev& m, const double* mom0, double* g, int* flags, cudaStream_t st) {
-  static const int sms = [] {
-    int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) n = 0;
-    return n;
-  }();
-  cudaError_t e = raise_smem_limit<k_mf_solve>();
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess) e = raise_smem_limit<k_mf_solve>();
   if (e != cudaSuccess) return e;
   // v and the staged rows: about 50 KB, so two CTAs fit an SM (one if the largest front is very wide)
   const size_t sm = 8 * ((size_t)m.max_f + (size_t)m.mcap);
