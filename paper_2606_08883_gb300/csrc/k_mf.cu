@@ -383,6 +383,9 @@ cudaError_t launch_mf_factor(const MfDev& m, const Plan& P, const double* ab, in
       count_launch(1);
       const int rounds = (int)((np_one * np_one + MF_THREADS - 1) / MF_THREADS);
       const size_t sm = 8 * (6 * (np_one + 1) + 1);
+      // R rounds of MF_THREADS entries: 36 and 64 (blocks of 81 to 128 unknowns that no cluster takes) fill the
+      // 255 registers of a thread and spill 912 and 480 bytes of them around the assembly and the division; still
+      // ahead of the block in shared memory (set-up with blocks of 90 unknowns 1.40 -> 1.12 ms, of 126 2.48 -> 1.92)
 #define MRCM_MF_FRONT(R) k_mf_front<R><<<nf, MF_THREADS, sm, st>>>(m, ab, P.mf_level[L], flags)
       if (rounds <= 2) MRCM_MF_FRONT(2);
       else if (rounds <= 4) MRCM_MF_FRONT(4);
