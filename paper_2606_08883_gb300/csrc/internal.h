@@ -37,7 +37,7 @@ struct MfItem {
   int front, u0, u1, p0, p1, vo;
 };
 constexpr int MF_LEAF = 16;       // leaf rectangles of at most this many subdomains
-constexpr int MF_MAX_NP = 128;    // largest pivot block (its inverse is formed in shared memory)
+constexpr int MF_MAX_NP = 128;    // largest pivot block (its inverse is formed in the registers of a CTA or cluster)
 constexpr int MF_TILE = 16;       // tile of the D, B and S products
 constexpr int MF_PARTS = 304;     // parts per level that the solve aims at (two CTAs on each of 152 SMs)
 constexpr int MF_PART_ROWS = 8;   // rows below which a part is not split further
@@ -82,7 +82,7 @@ struct Plan {
   std::vector<int> mf_rhs;         // per unknown the two side moments of its right-hand side (~ on the second: subtracted)
   size_t mf_vbuf = 0;              // doubles of the parts' v_P
   int mf_wslots = 0;               // upward message slots (sum of nu)
-  int mf_max_np = 0, mf_max_f = 0;
+  int mf_max_f = 0;
   int mf_mcap = 0;                 // largest staged part (doubles, padded rows), at most MF_STAGE
 };
 
@@ -286,7 +286,6 @@ cudaError_t launch_schwarz(const Geo& g, const void* Linv, int LS, bool fp32, co
                            double* zout, int* flags, int colour, cudaStream_t st, const float* in32 = nullptr);
 cudaError_t launch_reconstruct(const Geo& g, const double* psi0, const double* psi, const int* coff,
                                const double* c, double* z, cudaStream_t st);
-size_t factor_smem_bytes(int w, bool fp32, int nch);
 
 // coupling system (k_coarse.cu)
 struct CoarseDev {

@@ -143,8 +143,7 @@ __device__ __forceinline__ void tri_advance(int& i, int& j, int step) {
 // the thread that updates it), L^-1 by elimination on the identity, and S^-1 = L^-T L^-1.  The
 // scaled column of L (Cholesky) and the scaled row of L^-1 are written before the updates that
 // read them (two barriers per column), so every update entry is one FMA.
-template <typename T>
-__global__ void __launch_bounds__(256) k_factor(Geo g, int kind, int LS, T* __restrict__ Linv, int* flags, int nch) {
+__global__ void __launch_bounds__(256) k_factor(Geo g, int kind, int LS, float* __restrict__ Linv, int* flags, int nch) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int s = blockIdx.x;
   const bool ohat = kind != BOX_OMEGA_ROBIN;
@@ -156,19 +155,19 @@ __global__ void __launch_bounds__(256) k_factor(Geo g, int kind, int LS, T* __re
   const int tid = threadIdx.x, nt = blockDim.x;
   const int nth = nt / nch, half = tid / nth, tidh = tid - half * nth;
   const size_t per = 4 * (size_t)w * w + 4 * (size_t)w;   // one recursion's working arrays
-  T* Sm = reinterpret_cast<T*>(smem_raw) + half * per;   // Schur complement, then inverse work rows
-  T* Lm = Sm + w * w;                      // Cholesky factor of the line block
-  T* Lc = Lm + w * w;                      // L_JJ^-1 of the current line
-  T* Sp = Lc + w * w;                      // S^-1 of the previous (then current) line, lower part
-  T* ev = Sp + w * w;                      // couplings to the previous line
-  T* rinv = ev + w;                        // reciprocal diagonal of Lm
-  T* ev2 = rinv + w;                       // second coupling vector (middle line)
+  float* Sm = reinterpret_cast<float*>(smem_raw) + half * per;   // Schur complement, then inverse work rows
+  float* Lm = Sm + w * w;                      // Cholesky factor of the line block
+  float* Lc = Lm + w * w;                      // L_JJ^-1 of the current line
+  float* Sp = Lc + w * w;                      // S^-1 of the previous (then current) line, lower part
+  float* ev = Sp + w * w;                      // couplings to the previous line
+  float* rinv = ev + w;                        // reciprocal diagonal of Lm
+  float* ev2 = rinv + w;                       // second coupling vector (middle line)
   // the bottom recursion's last S^-1, read by the middle line when nch = 2
-  const T* Sp_bot = reinterpret_cast<T*>(smem_raw) + (nch == 2 ? per : 0) + 3 * (size_t)w * w;
+  const float* Sp_bot = reinterpret_cast<float*>(smem_raw) + (nch == 2 ? per : 0) + 3 * (size_t)w * w;
   __shared__ int bad;
   if (tid == 0) bad = 0;
-  T* out = Linv + (size_t)s * box_stride(w, h, LS);
-  T* ec_out = out + (size_t)h * LS;        // line couplings E_J[x], read by every solve
+  float* out = Linv + (size_t)s * box_stride(w, h, LS);
+  float* ec_out = out + (size_t)h * LS;        // line couplings E_J[x], read by every solve
   const int npk = w * (w + 1) / 2;
   const int iters = nch == 2 ? (m > h - 1 - m ? m : h - 1 - m) + 1 : h;
   for (int it = 0; it < iters; ++it) {
@@ -197,31 +196,31 @@ __global__ void __launch_bounds__(256) k_factor(Geo g, int kind, int LS, T* __re
       for (int i = tidh; i < w; i += nth) {
         double d, o, e;
         line_coeffs(g, b, robin, J, i, d, o, e, rt, rl);
-        ec_out[(size_t)J * w + i] = (T)e;
-        Sm[i * w + i] = (T)d;
-        if (i + 1 < w) Sm[(i + 1) * w + i] = (T)(-o);
+        ec_out[(size_t)J * w + i] = (float)e;
+        Sm[i * w + i] = (float)d;
+        if (i + 1 < w) Sm[(i + 1) * w + i] = (float)(-o);
         if (top) {
-          ev[i] = (T)e;
+          ev[i] = (float)e;
         } else if (bottom) {
           double d2, o2, e2;
           line_coeffs(g, b, robin, J + 1, i, d2, o2, e2, rt, rl);
-          ev[i] = (T)e2;
+          ev[i] = (float)e2;
         } else {
-          ev[i] = (T)e;                      // E_m (towards line m-1)
+          ev[i] = (float)e;                      // E_m (towards line m-1)
           double d2, o2, e2 = 0.0;
           if (J + 1 < h) line_coeffs(g, b, robin, J + 1, i, d2, o2, e2, rt, rl);
-          ev2[i] = (T)e2;                    // E_{m+1} (towards line m+1)
+          ev2[i] = (float)e2;                    // E_{m+1} (towards line m+1)
         }
       }
     __syncthreads();
     if (active) {
       const bool mid_up = mid && m > 0;          // S_{m-1}^-1: own Sp (nch = 2) or the stored top line
       const bool mid_dn = mid && m + 1 < h;      // S_{m+1}^-1: the bottom recursion's Sp
-      const T* Sup = out + (size_t)(m > 0 ? m - 1 : 0) * LS;
+      const float* Sup = out + (size_t)(m > 0 ? m - 1 : 0) * LS;
       int i, j;
       tri_at(tidh, i, j);
       for (int k = tidh; k < npk; k += nth, tri_advance(i, j, nth)) {
-        T v = (i == j || i == j + 1) ? Sm[i * w + j] : (T)0;
+        float v = (i == j || i == j + 1) ? Sm[i * w + j] : 0.0f;
         if (has_prev) v -= ev[i] * ev[j] * Sp[i * w + j];
         if (mid_up) v -= ev[i] * ev[j] * (nch == 2 ? Sp[i * w + j] : Sup[k]);
         if (mid_dn) v -= ev2[i] * ev2[j] * (nch == 2 ? Sp_bot[i * w + j] : Sp[i * w + j]);
@@ -231,21 +230,21 @@ __global__ void __launch_bounds__(256) k_factor(Geo g, int kind, int LS, T* __re
     __syncthreads();
     // (2) Cholesky of S_J: right-looking, column k of L written to Lm, trailing update in Sm
     if (active && tidh == 0) {
-      T p = Sm[0];
-      if (!(p > (T)0) || !isfinite((double)p)) {
+      float p = Sm[0];
+      if (!(p > 0.0f) || !isfinite((double)p)) {
         bad = 1;
-        p = (T)1;
+        p = 1.0f;
       }
-      const T d = sqrt(p);
+      const float d = sqrt(p);
       Lm[0] = d;
-      rinv[0] = (T)1 / d;
+      rinv[0] = 1.0f / d;
     }
     __syncthreads();
     for (int k = 0; k < w; ++k) {
       // column k of L first (one barrier), then the trailing update with one FMA per entry
       const int mm = w - k - 1;
       if (active) {
-        const T rd = rinv[k];
+        const float rd = rinv[k];
         for (int i = tidh; i < mm; i += nth) Lm[(k + 1 + i) * w + k] = Sm[(k + 1 + i) * w + k] * rd;
       }
       __syncthreads();
@@ -255,17 +254,17 @@ __global__ void __launch_bounds__(256) k_factor(Geo g, int kind, int LS, T* __re
         tri_at(tidh, ii, jj);
         for (int t = tidh; t < nup; t += nth, tri_advance(ii, jj, nth)) {
           const int i = k + 1 + ii, j = k + 1 + jj;
-          const T v = Sm[i * w + j] - Lm[i * w + k] * Lm[j * w + k];
+          const float v = Sm[i * w + j] - Lm[i * w + k] * Lm[j * w + k];
           Sm[i * w + j] = v;
           if (t == 0) {  // the next diagonal: its square root for column k + 1
-            T p = v;
-            if (!(p > (T)0) || !isfinite((double)p)) {
+            float p = v;
+            if (!(p > 0.0f) || !isfinite((double)p)) {
               bad = 1;
-              p = (T)1;
+              p = 1.0f;
             }
-            const T d = sqrt(p);
+            const float d = sqrt(p);
             Lm[(k + 1) * w + k + 1] = d;
-            rinv[k + 1] = (T)1 / d;
+            rinv[k + 1] = 1.0f / d;
           }
         }
       }
@@ -275,13 +274,13 @@ __global__ void __launch_bounds__(256) k_factor(Geo g, int kind, int LS, T* __re
     if (active)
       for (int k = tidh; k < w * w; k += nth) {
         const int i = k / w, j = k - i * w;
-        Sm[k] = (i == j) ? (T)1 : (T)0;
+        Sm[k] = (i == j) ? 1.0f : 0.0f;
       }
     __syncthreads();
     for (int k = 0; k < w; ++k) {
       // row k of L^-1 first (one barrier), then the rows below with one FMA per entry
       if (active) {
-        const T rk = rinv[k];
+        const float rk = rinv[k];
         for (int c = tidh; c <= k; c += nth) Lc[k * w + c] = Sm[k * w + c] * rk;
       }
       __syncthreads();
@@ -304,7 +303,7 @@ __global__ void __launch_bounds__(256) k_factor(Geo g, int kind, int LS, T* __re
       tri_advance(i1, j1, nth);
       for (int k = tidh; k < npk; k += 2 * nth) {
         const bool two = k + nth < npk;
-        T a0 = 0, a1 = 0;
+        float a0 = 0, a1 = 0;
         if (two) {
           // the second entry follows the first in packed order, so i1 >= i0: the first entry's
           // head, then both together (each summed in increasing q, as a single sum would be)
@@ -770,18 +769,9 @@ cudaError_t launch_line_coef(const Geo& g, int kind, double* coef, cudaStream_t 
   return cudaGetLastError();
 }
 
-size_t factor_smem_bytes(int w, bool fp32, int nch) {
-  const size_t e = fp32 ? 4 : 8;
-  return e * nch * (4 * (size_t)w * w + 4 * (size_t)w) + 16;
-}
-
 cudaError_t launch_factor(const Geo& g, int kind, int w, int hgt, int LS, void* Linv, bool fp32, int* flags,
                           cudaStream_t st, double* coef) {
   (void)hgt;
-  const int S = g.mx * g.my;
-  // both recursions at once when two sets of working arrays still leave room for two CTAs per SM
-  const int nch = factor_smem_bytes(w, fp32, 2) <= 112 * 1024 ? 2 : 1;
-  const size_t sm = factor_smem_bytes(w, fp32, nch);
   if (fp32 && w <= 36) {   // register-resident sweep, box width padded to a multiple of 4
     // it reads the Robin faces' t_R from the box tables only (k_robin_tab, formed with the assembly)
     if ((kind == BOX_OHAT_ROBIN && !g.rto) || (kind == BOX_OMEGA_ROBIN && !g.rtl)) return cudaErrorInvalidValue;
@@ -798,9 +788,12 @@ cudaError_t launch_factor(const Geo& g, int kind, int w, int hgt, int LS, void* 
     if (e != cudaSuccess) return e;
   }
   if (fp32) {
-    const cudaError_t e = raise_smem_limit<k_factor<float>>();
+    const cudaError_t e = raise_smem_limit<k_factor>();
     if (e != cudaSuccess) return e;
-    k_factor<float><<<S, 256, sm, st>>>(g, kind, LS, (float*)Linv, flags, nch);
+    // both recursions at once when two sets of working arrays still leave room for two CTAs per SM
+    const auto smem = [w](int nch) { return sizeof(float) * nch * (4 * (size_t)w * w + 4 * (size_t)w) + 16; };
+    const int nch = smem(2) <= 112 * 1024 ? 2 : 1;
+    k_factor<<<g.mx * g.my, 256, smem(nch), st>>>(g, kind, LS, (float*)Linv, flags, nch);
     count_launch(1);
   } else {
     double* L = (double*)Linv;

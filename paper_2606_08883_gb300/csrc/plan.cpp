@@ -249,7 +249,7 @@ static bool plan_mf(Plan& P) {
   P.mf_asm.clear();
   size_t fo = 0;
   int wo = 0;
-  P.mf_max_np = P.mf_max_f = 0;
+  P.mf_max_f = 0;
   P.mf_inv.assign(2 * P.mf_idx.size(), -1);
   for (int f = 0; f < nf; ++f) {
     MfFront& fr = P.mf_front[f];
@@ -277,7 +277,6 @@ static bool plan_mf(Plan& P) {
     fo += (size_t)fs * fs + 2 * (size_t)fr.nu * fr.np;
     fr.wo = wo;
     wo += fr.nu;
-    P.mf_max_np = std::max(P.mf_max_np, fr.np);
     P.mf_max_f = std::max(P.mf_max_f, fs);
   }
   P.mf_fbuf = fo;
