@@ -365,13 +365,13 @@ def phase_model(prob, q, prec):
 
 
 # DRAM traffic per launch (dram__bytes_read.sum + dram__bytes_write.sum) from one ncu --set full
-# capture of the kernel behind a phase, valid only while the kernel's source file is unchanged (its
-# SHA-256 at capture time); see profiles/ for the capture commands.
+# capture of the kernel behind a phase, valid only while the kernel's source file and common.cuh, whose
+# device functions it uses, are unchanged (kernel_sha at capture time); see profiles/ for the capture commands.
 NCU_TRAFFIC = {
-    ("schwarz", "fp32"): (560.455936e6 + 26.21568e6, "paper_2606_08883_gb300/csrc/k_local.cu",
-                          "90f92eb54507d866c4ceeca289bf9899587b21261f4891f4c94873720df18e60"),
-    ("factor_ohat_robin", "fp32"): (76.70784e6 + 353.64608e6, "paper_2606_08883_gb300/csrc/k_local.cu",
-                                    "90f92eb54507d866c4ceeca289bf9899587b21261f4891f4c94873720df18e60"),
+    ("schwarz", "fp32"): (561.02272e6 + 26.108672e6, "paper_2606_08883_gb300/csrc/k_local.cu",
+                          "30cdc36ac0aa973765a34eee0fdc2b4d843a6e4c0d89a75ca947273abb57bf39"),
+    ("factor_ohat_robin", "fp32"): (76.110336e6 + 353.747712e6, "paper_2606_08883_gb300/csrc/k_local.cu",
+                                    "30cdc36ac0aa973765a34eee0fdc2b4d843a6e4c0d89a75ca947273abb57bf39"),
 }
 
 
@@ -379,16 +379,24 @@ NCU_TRAFFIC = {
 # to the solve's average launch by the model's algorithmic bytes (krylov_model), in which the basis
 # sweeps that make the traffic grow in proportion.
 NCU_TRAFFIC_KRYLOV = (576.487936e6 + 62.679296e6, 5, "paper_2606_08883_gb300/csrc/k_krylov.cu",
-                      "e099eb7516a47ab82e145cb0b416229ac51b754d7435b4700501d691d76d788f")
+                      "7e078b729f6da38e5cf036bd278f5b4012cb0357de9167d14112d1a987f16aa3")
+
+
+def kernel_sha(src):
+    """SHA-256 over a kernel's source file and common.cuh beside it (None if either cannot be read)."""
+    d = hashlib.sha256()
+    for path in (src, os.path.join(os.path.dirname(src), "common.cuh")):
+        try:
+            with open(os.path.join(ROOT, path), "rb") as fh:
+                d.update(fh.read())
+        except OSError:
+            return None
+    return d.hexdigest()
 
 
 def krylov_traffic(n, iterations, restart):
     nbytes, jcap, src, sha = NCU_TRAFFIC_KRYLOV
-    try:
-        with open(os.path.join(ROOT, src), "rb") as fh:
-            if hashlib.sha256(fh.read()).hexdigest() != sha:
-                return None
-    except OSError:
+    if kernel_sha(src) != sha:
         return None
     at_cap = (2 * (jcap + 1) + 4) * 8 * n
     return nbytes * krylov_model(n, iterations, restart)[1] / at_cap
@@ -399,12 +407,7 @@ def ncu_traffic(name, prec):
     if entry is None:
         return None
     nbytes, src, sha = entry
-    try:
-        with open(os.path.join(ROOT, src), "rb") as fh:
-            cur = hashlib.sha256(fh.read()).hexdigest()
-    except OSError:
-        return None
-    return nbytes if cur == sha else None
+    return nbytes if kernel_sha(src) == sha else None
 
 
 def fp64_peak(peaks):
